@@ -296,11 +296,17 @@ loops_status upload_value_maps(loops_plan_s* p, const std::vector<int64_t>* rema
   }
   m.n_csr = (int64_t)csr_src.size();
   m.n_slots = n_slots;
+  m.wide = value_maps_wide(nnz, n_slots);
+  auto up = [&](void** dst, const std::vector<int64_t>& v) -> loops_status {
+    if (m.wide) return dev_upload((int64_t**)dst, v.data(), v.size(), m.bytes);
+    const std::vector<int32_t> w(v.begin(), v.end());
+    return dev_upload((int32_t**)dst, w.data(), w.size(), m.bytes);
+  };
   loops_status st;
-  if ((st = dev_upload(&m.csr_src, csr_src.data(), csr_src.size(), m.bytes))) return st;
+  if ((st = up(&m.csr_src, csr_src))) return st;
   if (n_slots) {
-    if ((st = dev_upload(&m.bcsr_ptr, cnt.data(), cnt.size(), m.bytes))) return st;
-    if ((st = dev_upload(&m.bcsr_src, bsrc.data(), bsrc.size(), m.bytes))) return st;
+    if ((st = up(&m.bcsr_ptr, cnt))) return st;
+    if ((st = up(&m.bcsr_src, bsrc))) return st;
   }
   return LOOPS_OK;
 }

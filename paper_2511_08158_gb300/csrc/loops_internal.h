@@ -203,13 +203,17 @@ struct SddmmDev {
 // Device maps from A's input entries to the stored values, for loops_plan_set_values:
 // CSR position p of the device value array takes input entry csr_src[p]; BCSR fragment slot f
 // takes the sum (in input order) of input entries bcsr_src[bcsr_ptr[f] .. bcsr_ptr[f+1]).
+// The maps hold 32-bit indices (half the bytes of the refresh's largest stream) unless the matrix
+// has 2^31 entries or fragment slots or more (`wide`: 64-bit).
 struct ValueMapDev {
   int64_t n_csr = 0, n_slots = 0;
-  int64_t* csr_src = nullptr;
-  int64_t* bcsr_ptr = nullptr;
-  int64_t* bcsr_src = nullptr;
+  bool wide = false;
+  void* csr_src = nullptr;
+  void* bcsr_ptr = nullptr;
+  void* bcsr_src = nullptr;
   int64_t bytes = 0;
 };
+inline bool value_maps_wide(int64_t nnz, int64_t n_slots) { return nnz > INT32_MAX || n_slots > INT32_MAX; }
 
 // Device descriptor of one matrix of a batched plan (pointers into its sub-plan, plus the
 // dense operands of the current call).

@@ -691,6 +691,10 @@ __global__ void item_gather_k(const int64_t* order, int64_t n, const int64_t* pr
   }
 }
 
+__global__ void narrow_k(const int64_t* in, int64_t n, int32_t* out) {
+  GS_LOOP(i, n) out[i] = (int32_t)in[i];
+}
+
 // ------------------------------------------------------------------ 6. backward pieces
 __global__ void sddmm_count_k(const int64_t* rp, int64_t n_rows, int64_t L, int64_t* n_items) {
   GS_LOOP(i, n_rows) {
@@ -1208,19 +1212,25 @@ loops_status build_part_device(loops_plan_s* p, const DevCsrIn& A, const int64_t
     free_value_maps(m);
     m.n_csr = n_csr_src;
     m.n_slots = n_fslots;
-    if (n_csr_src) {
-      TRY(own(&m.csr_src, n_csr_src, m.bytes));
-      TRY(cudaMemcpyAsync(m.csr_src, csr_src, (size_t)n_csr_src * 8, cudaMemcpyDeviceToDevice, s));
-    }
+    m.wide = value_maps_wide(nnz, n_fslots);
+    // owned copies, narrowed to 32 bits where they fit
+    auto keep_map = [&](void** dst, const int64_t* src, int64_t count) -> cudaError_t {
+      if (count <= 0) return cudaSuccess;
+      if (m.wide) {
+        cudaError_t e = own((int64_t**)dst, count, m.bytes);
+        return e != cudaSuccess ? e : cudaMemcpyAsync(*dst, src, (size_t)count * 8, cudaMemcpyDeviceToDevice, s);
+      }
+      cudaError_t e = own((int32_t**)dst, count, m.bytes);
+      if (e != cudaSuccess) return e;
+      narrow_k<<<grid_for(count), kThreads, 0, s>>>(src, count, (int32_t*)*dst);
+      return cudaGetLastError();
+    };
+    TRY(keep_map(&m.csr_src, csr_src, n_csr_src));
     if (n_fslots) {
       int64_t n_src = 0;
       TRY(to_host(&n_src, slot_ptr + n_fslots, s));
-      TRY(own(&m.bcsr_ptr, n_fslots + 1, m.bytes));
-      TRY(cudaMemcpyAsync(m.bcsr_ptr, slot_ptr, (size_t)(n_fslots + 1) * 8, cudaMemcpyDeviceToDevice, s));
-      if (n_src) {
-        TRY(own(&m.bcsr_src, n_src, m.bytes));
-        TRY(cudaMemcpyAsync(m.bcsr_src, slot_src, (size_t)n_src * 8, cudaMemcpyDeviceToDevice, s));
-      }
+      TRY(keep_map(&m.bcsr_ptr, slot_ptr, n_fslots + 1));
+      TRY(keep_map(&m.bcsr_src, slot_src, n_src));
     }
     p->has_vmap = true;
   }
