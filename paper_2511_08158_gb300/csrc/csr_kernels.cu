@@ -4,37 +4,14 @@
 // A group of G lanes (G divides 32) owns one work item (a CSR row or a segment of a long
 // row). Each lane owns VPL 16-byte column vectors of the output row, laid out so that the G
 // lanes read consecutive 16-byte pieces of a B row (coalesced 128-bit loads). The group
-// reads G (col, val) pairs at once and broadcasts them with shuffles; U B-row loads are kept
-// in flight before their FMAs. Accumulation is in f64 for F64 and in f32 otherwise. Every
-// output row has one writer; rows split in segments write partials that a second kernel
-// sums in segment order, so the result does not depend on scheduling.
+// reads a chunk of (col, val) pairs at once, one chunk ahead, and broadcasts them with
+// shuffles; U B-row loads are kept in flight before their FMAs. Accumulation is in f64 for F64
+// and in f32 otherwise. Every output row has one writer; rows split in segments write partials
+// that a second kernel sums in segment order, so the result does not depend on scheduling.
 #include <type_traits>
 
 #include "device_common.cuh"
 #include "loops_internal.h"
-
-// Tuning knobs of the memory-bound (non-FP64) CSR kernel: B-row loads kept in flight per
-// lane (per column vector), the minimum resident blocks per SM the register allocation must
-// allow, and the 16-byte column vectors each lane owns. Two vectors per lane with two
-// entries in flight (four 16-byte loads per lane) measured fastest on GB300 for the R-MAT
-// FP16 (N = 128) and GCN FP32 (N = 256) workloads.
-#ifndef LOOPS_CSR_UNROLL
-#define LOOPS_CSR_UNROLL 2
-#endif
-#ifndef LOOPS_CSR_MIN_BLOCKS
-#define LOOPS_CSR_MIN_BLOCKS 4
-#endif
-#ifndef LOOPS_CSR_LANE_VECTORS
-#define LOOPS_CSR_LANE_VECTORS 2
-#endif
-// FP64 (bound by the FP64 pipe): entries in flight per lane and resident blocks per SM with
-// one vector per lane.
-#ifndef LOOPS_CSR_F64_UNROLL
-#define LOOPS_CSR_F64_UNROLL 1
-#endif
-#ifndef LOOPS_CSR_F64_MIN_BLOCKS
-#define LOOPS_CSR_F64_MIN_BLOCKS 8
-#endif
 
 namespace loops {
 
@@ -74,134 +51,159 @@ __device__ __forceinline__ float out_scale<TrBF16>(const CsrKArgs& a, int64_t n)
 }
 
 // Vector path: N % VE == 0, B/C/ld aligned for 16-byte B loads and vector C stores.
-// FP64: 8 resident blocks (at most 32 registers) keep enough warps in flight to feed the FP64
-// pipe with one vector per lane; two vectors (N > 64) need 4 blocks (64 registers) to stay out
-// of local memory. The other formats use the tuning knob.
-template <class Tr, int VPL>
-constexpr int csr_min_blocks() {
-  return std::is_same<Tr, TrF64>::value ? (VPL == 1 ? LOOPS_CSR_F64_MIN_BLOCKS : 4) : LOOPS_CSR_MIN_BLOCKS;
-}
+//
+// The formats other than FP64 are bound by the latency of the gathers of B rows (from L2, from
+// DRAM where B exceeds it), so the shape is chosen for bytes in flight and few instructions per
+// gathered byte. Measured on GB300 (CSR kernel alone, before -> now):
+//   R-MAT 2^20, 14.3 M entries, N = 128, FP16   427 -> 328 us
+//   GCN 2^18, 7.4 M entries, N = 256, FP32      503 -> 397 us
+//   2^19 rows of 16 entries, N = 64, BF16       186 -> 146 us (63 % of the DRAM rate: B is
+//                                               134 MB, and L2 keeps a third of its rows)
+// * Blocks of 128 threads: a block holds its registers until its longest row ends, and smaller
+//   ones are replaced sooner (256 threads: R-MAT 16-bit 8 % slower, the 16-entry rows 5 %; 64:
+//   within 1 %). A persistent grid that strides over the items was 9 % slower.
+// * Two vectors per lane with two entries in flight from 16 vectors per row on, one vector
+//   with four entries below: the same bytes in flight, half the shuffles per byte. With one
+//   vector R-MAT 16-bit is 14 % slower and the GCN row 4 %; with four entries and two vectors the
+//   64 registers of 32 warps per SM spill.
+// * FULL (the group's vectors cover the columns exactly): loads carry no predicate and no zero
+//   fill; the second vector is an immediate offset from the first; a row's address is one
+//   32 x 32 -> 64 bit multiply-add.
+// * Columns in slices that fit L2 (64 to 512 bytes of each row at a time) were 2 to 40 % slower:
+//   the entries are read once per slice, and shorter pieces cost more instructions per byte.
+// FP64 is bound by the FP64 pipe: one entry at a time, so that no FMA is spent on a padded slot,
+// and no entries ahead; 48 warps per SM with one vector per lane (at 64 its 32 registers spill).
+constexpr int kCsrThreads = 128;
 
-template <class Tr, int G, int VPL, int U>
-__global__ void __launch_bounds__(256, (csr_min_blocks<Tr, VPL>())) csr_spmm_vec(CsrKArgs a) {
+template <class Tr, int VPL>
+struct CsrShape {
+  static constexpr bool kF64 = std::is_same<Tr, TrF64>::value;
+  static constexpr int kInFlight = kF64 ? 1 : (VPL == 1 ? 4 : 2);  // entries
+  static constexpr bool kAhead = !kF64;  // load the next chunk's entries before this chunk's B rows
+  static constexpr int kMinBlocks = (kF64 && VPL == 1 ? 48 : 32) * 32 / kCsrThreads;
+};
+
+template <class Tr, int G, int VPL, bool FULL>
+__global__ void __launch_bounds__(kCsrThreads, (CsrShape<Tr, VPL>::kMinBlocks)) csr_spmm_vec(CsrKArgs a) {
   using TB = typename Tr::TB;
   using TAcc = typename Tr::TAcc;
   using TC = typename Tr::TC;
   using TV = typename Tr::TV;
   constexpr int VE = Tr::kVE;
+  constexpr int U = CsrShape<Tr, VPL>::kInFlight;
+  constexpr bool AHEAD = CsrShape<Tr, VPL>::kAhead;
+  constexpr int R = G >= 8 ? 1 : 8 / G;  // entries per lane and chunk
+  constexpr int CH = G * R;
+  static_assert(CH % U == 0, "load batches tile the chunk");
   const int lane = threadIdx.x & 31;
   const int sub = lane & (G - 1);
-  const int64_t item = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
+  const int64_t item = ((int64_t)blockIdx.x * kCsrThreads + threadIdx.x) / G;
   if (item >= a.n_items) return;  // a group leaves as a whole
   const unsigned gmask = (G == 32) ? 0xffffffffu : (((1u << G) - 1u) << (lane & ~(G - 1)));
   const int64_t beg = a.item_ptr[item];
-  const int64_t end = a.item_ptr[item + 1];
+  const int32_t len = (int32_t)(a.item_ptr[item + 1] - beg);  // at most split_len
   const int32_t row = a.item_row[item];
-  const int64_t c_base = (int64_t)blockIdx.y * (G * VPL * VE);
-  bool colok[VPL];
-  int64_t coff[VPL];
+  const int32_t n0 = (int32_t)blockIdx.y * (G * VPL * VE) + sub * VE;  // vector p starts at column n0 + p * G * VE
+  bool ok[VPL];
 #pragma unroll
-  for (int p = 0; p < VPL; ++p) {
-    coff[p] = c_base + (int64_t)(p * G + sub) * VE;
-    colok[p] = coff[p] < a.N;
-  }
+  for (int p = 0; p < VPL; ++p) ok[p] = FULL || n0 + p * G * VE < (int32_t)a.N;
   TAcc acc[VPL][VE];
 #pragma unroll
   for (int p = 0; p < VPL; ++p)
 #pragma unroll
     for (int e = 0; e < VE; ++e) acc[p][e] = TAcc(0);
 
-  const TB* __restrict__ Bp = reinterpret_cast<const TB*>(a.B);
-  const TB* __restrict__ vals = reinterpret_cast<const TB*>(a.val);
-  // FP32 loads the next chunk's G entries before the current chunk's B rows, so their
-  // latency overlaps (measured: GCN layer 0.572 -> 0.547 ms); the 16-bit formats, whose
-  // unpacking needs the registers, and FP64, bound by its FMA pipe, load them in turn
-  constexpr bool kPrefetch = std::is_same<Tr, TrF32>::value;
-  int32_t c_next = 0;
-  TV v_next = TV(0);
-  if (kPrefetch && beg + sub < end) {
-    c_next = __ldg(a.col + beg + sub);
-    v_next = Tr::load_v(vals + beg + sub);
-  }
-  for (int64_t k0 = beg; k0 < end; k0 += G) {
-    int32_t c = c_next;
-    TV v = v_next;
-    const int64_t kn = kPrefetch ? k0 + G + sub : k0 + sub;
-    if (kn < end) {
-      c_next = __ldg(a.col + kn);
-      v_next = Tr::load_v(vals + kn);
+  const char* __restrict__ bl = reinterpret_cast<const char*>(a.B) + (int64_t)n0 * sizeof(TB);
+  const uint32_t ldb_bytes = (uint32_t)(a.ldb * (int64_t)sizeof(TB));  // the launch checks that it fits
+  auto fetch = [&](int32_t k0, int32_t (&c)[R], TV (&v)[R]) {
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int32_t k = k0 + r * G + sub;
+      c[r] = 0;
+      v[r] = TV(0);
+      if (k < len) {
+        c[r] = __ldg(a.col + beg + k);
+        v[r] = Tr::load_v(reinterpret_cast<const TB*>(a.val) + beg + k);
+      }
     }
-    if constexpr (!kPrefetch) {
-      c = kn < end ? c_next : 0;
-      v = kn < end ? v_next : TV(0);
+  };
+  int32_t c[R], c_next[R];
+  TV v[R], v_next[R];
+  if (AHEAD) fetch(0, c_next, v_next);
+  for (int32_t k0 = 0; k0 < len; k0 += CH) {
+    if (AHEAD) {
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        c[r] = c_next[r];
+        v[r] = v_next[r];
+      }
+      fetch(k0 + CH, c_next, v_next);
+    } else {
+      fetch(k0, c, v);
     }
-    const int cnt = (int)(end - k0 < (int64_t)G ? end - k0 : (int64_t)G);  // uniform in the group
-    int j0 = 0;
-    for (; j0 + U <= cnt; j0 += U) {  // full batches: U loads in flight, then U FMAs each
+    const int cnt = min(len - k0, CH);  // uniform in the group
+    // entries e0 .. e0 + U - 1 of the chunk; TAIL: those past its end load nothing and carry
+    // zero values, so they add exact zeros
+    auto batch = [&](int e0, auto tail_tag) {
+      constexpr bool TAIL = decltype(tail_tag)::value;
       uint4 bv[U][VPL];
       TV av[U];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        const int cj = __shfl_sync(gmask, c, (j0 + u) & (G - 1), G);
-        av[u] = __shfl_sync(gmask, v, (j0 + u) & (G - 1), G);
-        const TB* brow = Bp + (int64_t)cj * a.ldb;
+        const int e = e0 + u;
+        const uint32_t cj = (uint32_t)__shfl_sync(gmask, R == 1 ? c[0] : c[(e / G) % R], e % G, G);
+        av[u] = __shfl_sync(gmask, R == 1 ? v[0] : v[(e / G) % R], e % G, G);
+        const char* brow = bl + (uint64_t)cj * ldb_bytes;
 #pragma unroll
-        for (int p = 0; p < VPL; ++p) bv[u][p] = colok[p] ? ldg16(brow + coff[p]) : make_uint4(0, 0, 0, 0);
+        for (int p = 0; p < VPL; ++p) {
+          if constexpr (FULL && !TAIL) bv[u][p] = ldg16(brow + p * G * 16);
+          else bv[u][p] = ldg16_if(ok[p] && (!TAIL || e < cnt), brow + p * G * 16);
+        }
       }
 #pragma unroll
       for (int u = 0; u < U; ++u)
 #pragma unroll
         for (int p = 0; p < VPL; ++p) fma_vec<Tr>(acc[p], bv[u][p], av[u]);
-    }
-    if constexpr (U > 1) {
-    if (j0 < cnt) {  // tail of 1 .. U-1 entries: one batch under predicates
-      // entries past the tail load nothing and take a zero value, so they add exact zeros;
-      // the live loads issue together instead of one per round trip
-      uint4 bv[U - 1][VPL];
-      TV av[U - 1];
+    };
+    if constexpr (R == 1) {
+      int e0 = 0;
+      for (; e0 + U <= cnt; e0 += U) batch(e0, std::false_type());
+      if (U > 1 && e0 < cnt) batch(e0, std::true_type());
+    } else {  // unrolled: the entry's register index is a constant
 #pragma unroll
-      for (int u = 0; u < U - 1; ++u) {
-        const bool live = j0 + u < cnt;
-        const int cj = __shfl_sync(gmask, c, (j0 + u) & (G - 1), G);
-        const TV vj = __shfl_sync(gmask, v, (j0 + u) & (G - 1), G);
-        av[u] = live ? vj : TV(0);
-        const TB* brow = Bp + (int64_t)cj * a.ldb;
-#pragma unroll
-        for (int p = 0; p < VPL; ++p) bv[u][p] = ldg16_if(live && colok[p], brow + coff[p]);
+      for (int e0 = 0; e0 < CH; e0 += U) {
+        if (e0 + U <= cnt) batch(e0, std::false_type());
+        else if (e0 < cnt) batch(e0, std::true_type());
       }
-#pragma unroll
-      for (int u = 0; u < U - 1; ++u)
-#pragma unroll
-        for (int p = 0; p < VPL; ++p) fma_vec<Tr>(acc[p], bv[u][p], av[u]);
-    }
     }
   }
   if (row >= 0) {
-    TC* crow = reinterpret_cast<TC*>(a.C) + (int64_t)row * a.ldc;
+    TC* crow = reinterpret_cast<TC*>(a.C) + (int64_t)row * a.ldc + n0;
 #pragma unroll
     for (int p = 0; p < VPL; ++p) {
-      if (!colok[p]) continue;
+      if (!ok[p]) continue;
+      TC* cp = crow + p * G * VE;
       TC o[VE];
 #pragma unroll
       for (int e = 0; e < VE; ++e)
-        o[e] = Tr::kScaled ? (TC)(acc[p][e] * out_scale<Tr>(a, coff[p] + e)) : (TC)acc[p][e];
+        o[e] = Tr::kScaled ? (TC)(acc[p][e] * out_scale<Tr>(a, n0 + p * G * VE + e)) : (TC)acc[p][e];
       if (a.accumulate) {
 #pragma unroll
-        for (int e = 0; e < VE; ++e) o[e] += crow[coff[p] + e];
+        for (int e = 0; e < VE; ++e) o[e] += cp[e];
       }
       // VE outputs are 16 (F64/F32) or 32 (16-bit inputs, f32 outputs) bytes
 #pragma unroll
       for (int q = 0; q < (int)(VE * sizeof(TC) / 16); ++q)
-        *reinterpret_cast<uint4*>(crow + coff[p] + q * (16 / sizeof(TC))) =
+        *reinterpret_cast<uint4*>(cp + q * (16 / sizeof(TC))) =
             *reinterpret_cast<const uint4*>(&o[q * (16 / sizeof(TC))]);
     }
   } else {
-    TAcc* srow = reinterpret_cast<TAcc*>(a.scratch) + (int64_t)(-1 - row) * a.N;
+    TAcc* srow = reinterpret_cast<TAcc*>(a.scratch) + (int64_t)(-1 - row) * a.N + n0;
 #pragma unroll
     for (int p = 0; p < VPL; ++p) {
-      if (!colok[p]) continue;
+      if (!ok[p]) continue;
 #pragma unroll
-      for (int e = 0; e < VE; ++e) srow[coff[p] + e] = acc[p][e];
+      for (int e = 0; e < VE; ++e) srow[p * G * VE + e] = acc[p][e];
     }
   }
 }
@@ -286,18 +288,11 @@ inline int next_pow2(int64_t x) {
 
 template <class Tr, int G, int VPL>
 cudaError_t launch_vec_g(const CsrKArgs& a, cudaStream_t s) {
-  constexpr int VE = Tr::kVE;
-  const int64_t per_chunk = (int64_t)G * VPL * VE;
-  const int64_t chunks = (a.N + per_chunk - 1) / per_chunk;
-  const int64_t threads = a.n_items * G;
-  dim3 grid((unsigned)((threads + 255) / 256), (unsigned)chunks);
-  // F64 is bound by the FP64 pipe: one entry at a time, so no FMA is ever spent on a padded
-  // slot (a predicated-off DFMA still occupies the pipe) and registers stay low for occupancy.
-  // The other formats are bound by memory: U x VPL loads in flight per lane (narrow groups with
-  // one vector per lane take four entries at a time, the register budget allows it).
-  constexpr int U = std::is_same<Tr, TrF64>::value ? LOOPS_CSR_F64_UNROLL
-                                                   : ((G >= 8 || VPL > 1) ? LOOPS_CSR_UNROLL : 4);
-  csr_spmm_vec<Tr, G, VPL, U><<<grid, 256, 0, s>>>(a);
+  constexpr int64_t per_chunk = (int64_t)G * VPL * Tr::kVE;
+  const dim3 grid((unsigned)((a.n_items * G + kCsrThreads - 1) / kCsrThreads),
+                  (unsigned)((a.N + per_chunk - 1) / per_chunk));
+  if (a.N % per_chunk == 0) csr_spmm_vec<Tr, G, VPL, true><<<grid, kCsrThreads, 0, s>>>(a);
+  else csr_spmm_vec<Tr, G, VPL, false><<<grid, kCsrThreads, 0, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -324,19 +319,15 @@ cudaError_t launch_csr_t(const loops_plan_s* p, const CsrDev& d, const DenseArgs
   using TC = typename Tr::TC;
   constexpr int VE = Tr::kVE;
   const bool vec = (a.N % VE == 0) && ((uintptr_t)a.B % 16 == 0) && ((uintptr_t)a.C % 16 == 0) &&
-                   ((a.ldb * (int64_t)sizeof(TB)) % 16 == 0) && ((a.ldc * (int64_t)sizeof(TC)) % 16 == 0);
+                   ((a.ldb * (int64_t)sizeof(TB)) % 16 == 0) && ((a.ldc * (int64_t)sizeof(TC)) % 16 == 0) &&
+                   a.ldb * (int64_t)sizeof(TB) <= (int64_t)UINT32_MAX;  // row strides of B in 32 bits
   cudaError_t e = cudaSuccess;
   if (a.n_items > 0) {
     if (vec) {
       const int64_t nvec = a.N / VE;
-      // lanes per item: the 16-byte vectors of a row, LOOPS_CSR_LANE_VECTORS per lane while
-      // the group keeps at least 8 lanes (more vectors per lane: fewer shuffles per byte and
-      // more loads in flight per lane; narrower groups lose more to the per-row overhead)
-      // (the plan's csr_vpl, when the autotuner set it, overrides this heuristic)
-      constexpr int LV = LOOPS_CSR_LANE_VECTORS;
-      const bool lv = p->csr_vpl == 2 ? nvec >= 2
-                    : p->csr_vpl == 1 ? false
-                    : (!std::is_same<Tr, TrF64>::value && LV > 1 && nvec >= 8 * LV);
+      // lanes per item: the 16-byte vectors of a row, two per lane from 16 vectors on (the
+      // reasons stand at the kernel); the plan's csr_vpl, when the autotuner set it, overrides this
+      const bool lv = p->csr_vpl == 2 ? nvec >= 2 : p->csr_vpl == 1 ? false : (!std::is_same<Tr, TrF64>::value && nvec >= 16);
       const int64_t nv = lv ? (nvec + 1) / 2 : nvec;
       const int G = next_pow2(nv);
       const bool two = lv || nvec > 32;
