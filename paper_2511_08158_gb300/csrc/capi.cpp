@@ -367,10 +367,8 @@ static loops_status check_dense(const void* ptr, int64_t rows, int64_t N, int64_
   return LOOPS_OK;
 }
 
-// Run C = A.B on the plan: BCSR part on the side stream, CSR part on `s`, joined by events.
-static loops_status run_spmm(loops_plan_s* p, const void* B, int64_t ldb, const float* col_scale,
-                             void* C, int64_t ldc, cudaStream_t s) {
-  if (p->n_rows == 0 || p->N == 0) return LOOPS_OK;
+static DenseArgs dense_args(const loops_plan_s* p, const void* B, int64_t ldb, const float* col_scale, void* C,
+                            int64_t ldc) {
   DenseArgs a;
   a.B = B;
   a.ldb = ldb;
@@ -381,6 +379,14 @@ static loops_status run_spmm(loops_plan_s* p, const void* B, int64_t ldb, const 
   a.inv_scale_f = (float)(1.0 / p->scale);
   a.N = p->N;
   a.n_rows = p->n_rows;
+  return a;
+}
+
+// Run C = A.B on the plan: BCSR part on the side stream, CSR part on `s`, joined by events.
+static loops_status run_spmm(loops_plan_s* p, const void* B, int64_t ldb, const float* col_scale,
+                             void* C, int64_t ldc, cudaStream_t s) {
+  if (p->n_rows == 0 || p->N == 0) return LOOPS_OK;
+  const DenseArgs a = dense_args(p, B, ldb, col_scale, C, ldc);
   const bool has_csr = p->dev.csr.n_items > 0;
   const bool has_bcsr = p->dev.bcsr.n_rb > 0;
   const bool tm = p->timing;
@@ -1236,6 +1242,12 @@ loops_status loops_spmm_backward_scaled(loops_plan_t p, const void* dC, int64_t 
   }
   if ((st = check_dense(dC, p->n_rows, p->N, lddc, "dC"))) return st;
   cudaStream_t s = (cudaStream_t)stream;
+  if (dB && dvals && p->nnz > 0 && csr_backward_applies(p, dC, lddc, B, ldb, dB, lddb)) {
+    if ((st = check_dense(dB, p->n_cols, p->N, lddb, "dB"))) return st;
+    if ((st = check_dense(B, p->n_cols, p->N, ldb, "B"))) return st;
+    const DenseArgs a = dense_args(p->transposed, dC, lddc, dc_scale, dB, lddb);
+    return cuda_status(launch_csr_backward(p, a, B, ldb, dvals, b_scale, s), "backward launch");
+  }
   if (dB) {
     if ((st = check_dense(dB, p->n_cols, p->N, lddb, "dB"))) return st;
     // dB = A^T . (dC diag(dc_scale)) = (A^T . dC) diag(dc_scale): the column scales of the

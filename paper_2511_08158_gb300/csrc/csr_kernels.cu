@@ -25,6 +25,7 @@ struct CsrKArgs {
   int64_t n_items;
   const void* B;
   int64_t ldb;
+  uint32_t ldb_bytes;    // vector paths only, whose launches check that it fits
   void* C;
   int64_t ldc;
   void* scratch;         // n_slots x N accumulators
@@ -48,6 +49,62 @@ __device__ __forceinline__ float out_scale<TrF16>(const CsrKArgs& a, int64_t n) 
 template <>
 __device__ __forceinline__ float out_scale<TrBF16>(const CsrKArgs& a, int64_t n) {
   return a.col_scale ? a.col_scale[n] * a.inv_scale_f : a.inv_scale_f;
+}
+
+// A chunk of an item's entries, R per lane (entry r * G + sub): columns and values, zeros past the
+// item's end.
+template <class Tr, int G, int R>
+__device__ __forceinline__ void fetch_entries(const CsrKArgs& a, int64_t beg, int32_t len, int32_t k0, int sub,
+                                              int32_t (&c)[R], typename Tr::TV (&v)[R]) {
+  using TB = typename Tr::TB;
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const int32_t k = k0 + r * G + sub;
+    c[r] = 0;
+    v[r] = 0;
+    if (k < len) {
+      c[r] = __ldg(a.col + beg + k);
+      v[r] = Tr::load_v(reinterpret_cast<const TB*>(a.val) + beg + k);
+    }
+  }
+}
+
+// Output of an item: its C row (scaled), or its slot of partial sums.
+template <class Tr, int G, int VPL>
+__device__ __forceinline__ void store_item(const CsrKArgs& a, int32_t row, int32_t n0, const bool (&ok)[VPL],
+                                           const typename Tr::TAcc (&acc)[VPL][Tr::kVE]) {
+  using TAcc = typename Tr::TAcc;
+  using TC = typename Tr::TC;
+  constexpr int VE = Tr::kVE;
+  if (row >= 0) {
+    TC* crow = reinterpret_cast<TC*>(a.C) + (int64_t)row * a.ldc + n0;
+#pragma unroll
+    for (int p = 0; p < VPL; ++p) {
+      if (!ok[p]) continue;
+      TC* cp = crow + p * G * VE;
+      TC o[VE];
+#pragma unroll
+      for (int e = 0; e < VE; ++e)
+        o[e] = Tr::kScaled ? (TC)(acc[p][e] * out_scale<Tr>(a, n0 + p * G * VE + e)) : (TC)acc[p][e];
+      if (a.accumulate) {
+#pragma unroll
+        for (int e = 0; e < VE; ++e) o[e] += cp[e];
+      }
+      // VE outputs are 16 (F64/F32) or 32 (16-bit inputs, f32 outputs) bytes
+#pragma unroll
+      for (int q = 0; q < (int)(VE * sizeof(TC) / 16); ++q)
+        *reinterpret_cast<uint4*>(cp + q * (16 / sizeof(TC))) =
+            *reinterpret_cast<const uint4*>(&o[q * (16 / sizeof(TC))]);
+    }
+  } else {
+    TAcc* srow = reinterpret_cast<TAcc*>(a.scratch) + (int64_t)(-1 - row) * a.N + n0;
+#pragma unroll
+    for (int p = 0; p < VPL; ++p) {
+      if (!ok[p]) continue;
+#pragma unroll
+      for (int e = 0; e < VE; ++e) srow[p * G * VE + e] = acc[p][e];
+    }
+  }
 }
 
 // Vector path: N % VE == 0, B/C/ld aligned for 16-byte B loads and vector C stores.
@@ -87,7 +144,6 @@ template <class Tr, int G, int VPL, bool FULL>
 __global__ void __launch_bounds__(kCsrThreads, (CsrShape<Tr, VPL>::kMinBlocks)) csr_spmm_vec(CsrKArgs a) {
   using TB = typename Tr::TB;
   using TAcc = typename Tr::TAcc;
-  using TC = typename Tr::TC;
   using TV = typename Tr::TV;
   constexpr int VE = Tr::kVE;
   constexpr int U = CsrShape<Tr, VPL>::kInFlight;
@@ -114,22 +170,9 @@ __global__ void __launch_bounds__(kCsrThreads, (CsrShape<Tr, VPL>::kMinBlocks)) 
     for (int e = 0; e < VE; ++e) acc[p][e] = TAcc(0);
 
   const char* __restrict__ bl = reinterpret_cast<const char*>(a.B) + (int64_t)n0 * sizeof(TB);
-  const uint32_t ldb_bytes = (uint32_t)(a.ldb * (int64_t)sizeof(TB));  // the launch checks that it fits
-  auto fetch = [&](int32_t k0, int32_t (&c)[R], TV (&v)[R]) {
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const int32_t k = k0 + r * G + sub;
-      c[r] = 0;
-      v[r] = TV(0);
-      if (k < len) {
-        c[r] = __ldg(a.col + beg + k);
-        v[r] = Tr::load_v(reinterpret_cast<const TB*>(a.val) + beg + k);
-      }
-    }
-  };
   int32_t c[R], c_next[R];
   TV v[R], v_next[R];
-  if (AHEAD) fetch(0, c_next, v_next);
+  if (AHEAD) fetch_entries<Tr, G>(a, beg, len, 0, sub, c_next, v_next);
   for (int32_t k0 = 0; k0 < len; k0 += CH) {
     if (AHEAD) {
 #pragma unroll
@@ -137,9 +180,9 @@ __global__ void __launch_bounds__(kCsrThreads, (CsrShape<Tr, VPL>::kMinBlocks)) 
         c[r] = c_next[r];
         v[r] = v_next[r];
       }
-      fetch(k0 + CH, c_next, v_next);
+      fetch_entries<Tr, G>(a, beg, len, k0 + CH, sub, c_next, v_next);
     } else {
-      fetch(k0, c, v);
+      fetch_entries<Tr, G>(a, beg, len, k0, sub, c, v);
     }
     const int cnt = min(len - k0, CH);  // uniform in the group
     // entries e0 .. e0 + U - 1 of the chunk; TAIL: those past its end load nothing and carry
@@ -153,7 +196,7 @@ __global__ void __launch_bounds__(kCsrThreads, (CsrShape<Tr, VPL>::kMinBlocks)) 
         const int e = e0 + u;
         const uint32_t cj = (uint32_t)__shfl_sync(gmask, R == 1 ? c[0] : c[(e / G) % R], e % G, G);
         av[u] = __shfl_sync(gmask, R == 1 ? v[0] : v[(e / G) % R], e % G, G);
-        const char* brow = bl + (uint64_t)cj * ldb_bytes;
+        const char* brow = bl + (uint64_t)cj * a.ldb_bytes;
 #pragma unroll
         for (int p = 0; p < VPL; ++p) {
           if constexpr (FULL && !TAIL) bv[u][p] = ldg16(brow + p * G * 16);
@@ -177,35 +220,7 @@ __global__ void __launch_bounds__(kCsrThreads, (CsrShape<Tr, VPL>::kMinBlocks)) 
       }
     }
   }
-  if (row >= 0) {
-    TC* crow = reinterpret_cast<TC*>(a.C) + (int64_t)row * a.ldc + n0;
-#pragma unroll
-    for (int p = 0; p < VPL; ++p) {
-      if (!ok[p]) continue;
-      TC* cp = crow + p * G * VE;
-      TC o[VE];
-#pragma unroll
-      for (int e = 0; e < VE; ++e)
-        o[e] = Tr::kScaled ? (TC)(acc[p][e] * out_scale<Tr>(a, n0 + p * G * VE + e)) : (TC)acc[p][e];
-      if (a.accumulate) {
-#pragma unroll
-        for (int e = 0; e < VE; ++e) o[e] += cp[e];
-      }
-      // VE outputs are 16 (F64/F32) or 32 (16-bit inputs, f32 outputs) bytes
-#pragma unroll
-      for (int q = 0; q < (int)(VE * sizeof(TC) / 16); ++q)
-        *reinterpret_cast<uint4*>(cp + q * (16 / sizeof(TC))) =
-            *reinterpret_cast<const uint4*>(&o[q * (16 / sizeof(TC))]);
-    }
-  } else {
-    TAcc* srow = reinterpret_cast<TAcc*>(a.scratch) + (int64_t)(-1 - row) * a.N + n0;
-#pragma unroll
-    for (int p = 0; p < VPL; ++p) {
-      if (!ok[p]) continue;
-#pragma unroll
-      for (int e = 0; e < VE; ++e) srow[p * G * VE + e] = acc[p][e];
-    }
-  }
+  store_item<Tr, G, VPL>(a, row, n0, ok, acc);
 }
 
 // Scalar path for any N and alignment: 32 lanes per item, one column per lane per pass.
@@ -280,6 +295,187 @@ __global__ void __launch_bounds__(256) split_reduce(const int32_t* __restrict__ 
   }
 }
 
+// Backward of C = A . B in one pass over A^T: dB[j, :] = sum_i a_ij dC[i, :] and
+// dvals[a_ij] = <dC[i, :], B[j, :]> read the same rows of dC, so the group that owns row j of A^T
+// keeps B[j, :] (times the column weights) beside its accumulators and takes both from each row
+// it gathers. The gathers of dC rows bound it as they bound the SpMM and the SDDMM that it
+// replaces, and are made once instead of twice. Measured on GB300 (dB and dvals together):
+//   GCN 2^18, 7.4 M entries, N = 256, FP32      930 -> 566 us
+//   the same graph, N = 128, BF16               369 -> 265 us
+// The shape is the SpMM's: 128 threads, entries one chunk ahead, no predicates where the group
+// covers the columns. Bytes in flight and warps decide: FP32 takes four entries in flight at 32
+// warps per SM (two: 10 % slower step; 24 warps: 5 %), the 16-bit formats two vectors per lane
+// from 16 on with two entries at 28 warps (one vector: 4 % slower step; 32 warps spill: 11 %).
+// The input entry of a dot product (`src`) is loaded with its column and value: loaded where
+// dvals is stored, it stalled every batch (20 % slower).
+template <class Tr, int VPL>
+struct BwdShape {
+  static constexpr bool kF64 = std::is_same<Tr, TrF64>::value, k16 = Tr::kVE == 8;
+  static constexpr int kInFlight = VPL == 2 && (k16 || kF64) ? 2 : 4;  // entries
+  static constexpr int kWarps = kF64 ? (VPL == 2 ? 16 : 24) : (k16 && VPL == 2 ? 28 : 32);
+};
+
+struct BwdKArgs {
+  const void* B;             // rows of B, one per row of A^T
+  int64_t ldb;
+  void* dvals;               // input order
+  const int32_t* src;        // input entry of every stored entry
+  const int32_t* split_row;  // rows cut into segments, and their slots
+  const int32_t* split_slot_ptr;
+  int64_t n_split;
+  const float* dc_scale;     // optional column scales of dC and B (16-bit dtypes)
+  const float* b_scale;
+};
+
+template <class Tr, int G, int VPL, bool FULL>
+__global__ void __launch_bounds__(kCsrThreads, (BwdShape<Tr, VPL>::kWarps * 32 / kCsrThreads))
+    csr_backward_vec(CsrKArgs a, BwdKArgs w) {
+  using TB = typename Tr::TB;
+  using TAcc = typename Tr::TAcc;
+  using TC = typename Tr::TC;
+  using TV = typename Tr::TV;
+  constexpr int VE = Tr::kVE;
+  constexpr int U = BwdShape<Tr, VPL>::kInFlight;
+  constexpr int R = G >= 8 ? 1 : 8 / G;  // entries per lane and chunk
+  constexpr int CH = G * R;
+  static_assert(CH % U == 0, "load batches tile the chunk");
+  const int lane = threadIdx.x & 31;
+  const int sub = lane & (G - 1);
+  const int64_t item = ((int64_t)blockIdx.x * kCsrThreads + threadIdx.x) / G;
+  if (item >= a.n_items) return;  // a group leaves as a whole
+  const unsigned gmask = (G == 32) ? 0xffffffffu : (((1u << G) - 1u) << (lane & ~(G - 1)));
+  const int64_t beg = a.item_ptr[item];
+  const int32_t len = (int32_t)(a.item_ptr[item + 1] - beg);
+  const int32_t row = a.item_row[item];
+  auto fetch = [&](int32_t k0, int32_t (&c)[R], TV (&v)[R], int32_t (&x)[R]) {
+    fetch_entries<Tr, G>(a, beg, len, k0, sub, c, v);
+#pragma unroll
+    for (int r = 0; r < R; ++r) x[r] = k0 + r * G + sub < len ? __ldg(w.src + beg + k0 + r * G + sub) : 0;
+  };
+  int32_t c_next[R], x_next[R];
+  TV v_next[R];
+  fetch(0, c_next, v_next, x_next);
+  int32_t j = row;
+  if (row < 0) {  // a segment: the split row that holds its slot
+    const int32_t slot = -1 - row;
+    int64_t lo = 0, hi = w.n_split;  // split_slot_ptr[lo] <= slot < split_slot_ptr[hi]
+    while (hi - lo > 1) {
+      const int64_t mid = (lo + hi) >> 1;
+      if (w.split_slot_ptr[mid] <= slot) lo = mid; else hi = mid;
+    }
+    j = w.split_row[lo];
+  }
+  const int32_t n0 = sub * VE;
+  bool ok[VPL];
+  TAcc acc[VPL][VE], bj[VPL][VE];
+#pragma unroll
+  for (int p = 0; p < VPL; ++p) {
+    const int32_t n = n0 + p * G * VE;
+    ok[p] = FULL || n < (int32_t)a.N;
+    unpack16<Tr>(ldg16_if(ok[p], reinterpret_cast<const TB*>(w.B) + (int64_t)j * w.ldb + n), bj[p]);
+    if constexpr (Tr::kScaled) {
+      if (ok[p]) {
+#pragma unroll
+        for (int e = 0; e < VE; ++e)
+          bj[p][e] *= (w.dc_scale ? w.dc_scale[n + e] : 1.f) * (w.b_scale ? w.b_scale[n + e] : 1.f);
+      }
+    }
+#pragma unroll
+    for (int e = 0; e < VE; ++e) acc[p][e] = TAcc(0);
+  }
+  const char* __restrict__ dl = reinterpret_cast<const char*>(a.B) + (int64_t)n0 * sizeof(TB);
+  TC* __restrict__ dvals = reinterpret_cast<TC*>(w.dvals);
+  for (int32_t k0 = 0; k0 < len; k0 += CH) {
+    int32_t c[R], x[R];
+    TV v[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      c[r] = c_next[r];
+      v[r] = v_next[r];
+      x[r] = x_next[r];
+    }
+    fetch(k0 + CH, c_next, v_next, x_next);
+    const int cnt = min(len - k0, CH);  // uniform in the group
+    // entries e0 .. e0 + U - 1 of the chunk; TAIL: those past its end load nothing, carry zero
+    // values and are not stored
+    auto batch = [&](int e0, auto tail_tag) {
+      constexpr bool TAIL = decltype(tail_tag)::value;
+      uint4 dv[U][VPL];
+      TV av[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int e = e0 + u;
+        const uint32_t i = (uint32_t)__shfl_sync(gmask, R == 1 ? c[0] : c[(e / G) % R], e % G, G);
+        av[u] = __shfl_sync(gmask, R == 1 ? v[0] : v[(e / G) % R], e % G, G);
+        const char* drow = dl + (uint64_t)i * a.ldb_bytes;
+#pragma unroll
+        for (int p = 0; p < VPL; ++p) {
+          if constexpr (FULL && !TAIL) dv[u][p] = ldg16(drow + p * G * 16);
+          else dv[u][p] = ldg16_if(ok[p] && (!TAIL || e < cnt), drow + p * G * 16);
+        }
+      }
+      TAcc s[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        s[u] = TAcc(0);
+#pragma unroll
+        for (int p = 0; p < VPL; ++p) {
+          TAcc d[VE];
+          unpack16<Tr>(dv[u][p], d);
+#pragma unroll
+          for (int e = 0; e < VE; ++e) s[u] = fma(bj[p][e], d[e], s[u]);
+          fma_vec<Tr>(acc[p], dv[u][p], av[u]);
+        }
+      }
+      // sums over the group in a fixed order. With at least U lanes a lane keeps half of the
+      // entries at each of the first steps, so that 1 / U of the group ends with one entry's sum
+      if constexpr (G >= U) {
+        TAcc t;
+        int mine;
+        if constexpr (U == 4) {
+          const bool h1 = (sub & (G / 2)) != 0, h2 = (sub & (G / 4)) != 0;
+          TAcc t0 = h1 ? s[2] : s[0], t1 = h1 ? s[3] : s[1];
+          t0 += __shfl_xor_sync(gmask, h1 ? s[0] : s[2], G / 2, G);
+          t1 += __shfl_xor_sync(gmask, h1 ? s[1] : s[3], G / 2, G);
+          t = h2 ? t1 : t0;
+          t += __shfl_xor_sync(gmask, h2 ? t0 : t1, G / 4, G);
+          mine = e0 + (h1 ? 2 : 0) + (h2 ? 1 : 0);
+        } else {
+          const bool h1 = (sub & (G / 2)) != 0;
+          t = h1 ? s[1] : s[0];
+          t += __shfl_xor_sync(gmask, h1 ? s[0] : s[1], G / 2, G);
+          mine = e0 + (h1 ? 1 : 0);
+        }
+#pragma unroll
+        for (int off = G / U / 2; off > 0; off >>= 1) t += __shfl_xor_sync(gmask, t, off, G);
+        const int32_t at = __shfl_sync(gmask, R == 1 ? x[0] : x[(e0 / G) % R], mine % G, G);
+        if ((sub & (G / U - 1)) == 0 && (!TAIL || mine < cnt)) dvals[at] = (TC)t;
+      } else {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          TAcc t = s[u];
+#pragma unroll
+          for (int off = G / 2; off > 0; off >>= 1) t += __shfl_xor_sync(gmask, t, off, G);
+          const int32_t at = __shfl_sync(gmask, x[((e0 + u) / G) % R], (e0 + u) % G, G);
+          if (sub == 0 && (!TAIL || e0 + u < cnt)) dvals[at] = (TC)t;
+        }
+      }
+    };
+    if constexpr (R == 1) {
+      int e0 = 0;
+      for (; e0 + U <= cnt; e0 += U) batch(e0, std::false_type());
+      if (e0 < cnt) batch(e0, std::true_type());
+    } else {  // unrolled: the entry's register index is a constant
+#pragma unroll
+      for (int e0 = 0; e0 < CH; e0 += U) {
+        if (e0 + U <= cnt) batch(e0, std::false_type());
+        else if (e0 < cnt) batch(e0, std::true_type());
+      }
+    }
+  }
+  store_item<Tr, G, VPL>(a, row, n0, ok, acc);
+}
+
 inline int next_pow2(int64_t x) {
   int p = 1;
   while (p < x && p < 32) p <<= 1;
@@ -296,9 +492,7 @@ cudaError_t launch_vec_g(const CsrKArgs& a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-template <class Tr>
-cudaError_t launch_csr_t(const loops_plan_s* p, const CsrDev& d, const DenseArgs& da, bool accumulate,
-                         cudaStream_t s) {
+CsrKArgs csr_args(const loops_plan_s* p, const CsrDev& d, const DenseArgs& da, bool accumulate) {
   CsrKArgs a;
   a.accumulate = accumulate ? 1 : 0;
   a.item_row = d.item_row;
@@ -308,6 +502,7 @@ cudaError_t launch_csr_t(const loops_plan_s* p, const CsrDev& d, const DenseArgs
   a.n_items = d.n_items;
   a.B = da.B;
   a.ldb = da.ldb;
+  a.ldb_bytes = (uint32_t)(da.ldb * dense_elem_bytes(p->dtype));
   a.C = da.C;
   a.ldc = da.ldc;
   a.scratch = d.scratch;
@@ -315,6 +510,21 @@ cudaError_t launch_csr_t(const loops_plan_s* p, const CsrDev& d, const DenseArgs
   a.inv_scale_f = da.inv_scale_f;
   a.inv_scale_d = da.inv_scale_d;
   a.N = da.N;
+  return a;
+}
+
+template <class Tr>
+cudaError_t launch_split_reduce(const CsrDev& d, const CsrKArgs& a, cudaStream_t s) {
+  if (d.n_split == 0) return cudaSuccess;
+  dim3 grid((unsigned)d.n_split, (unsigned)std::min<int64_t>((a.N + 255) / 256, 64));
+  split_reduce<Tr><<<grid, 256, 0, s>>>(d.split_row, d.split_slot_ptr, d.n_split, a);
+  return cudaGetLastError();
+}
+
+template <class Tr>
+cudaError_t launch_csr_t(const loops_plan_s* p, const CsrDev& d, const DenseArgs& da, bool accumulate,
+                         cudaStream_t s) {
+  const CsrKArgs a = csr_args(p, d, da, accumulate);
   using TB = typename Tr::TB;
   using TC = typename Tr::TC;
   constexpr int VE = Tr::kVE;
@@ -345,15 +555,74 @@ cudaError_t launch_csr_t(const loops_plan_s* p, const CsrDev& d, const DenseArgs
       e = cudaGetLastError();
     }
   }
-  if (e == cudaSuccess && d.n_split > 0) {
-    dim3 grid((unsigned)d.n_split, (unsigned)std::min<int64_t>((a.N + 255) / 256, 64));
-    split_reduce<Tr><<<grid, 256, 0, s>>>(d.split_row, d.split_slot_ptr, d.n_split, a);
-    e = cudaGetLastError();
-  }
+  if (e == cudaSuccess) e = launch_split_reduce<Tr>(d, a, s);
   return e;
 }
 
+template <class Tr>
+cudaError_t launch_csr_backward_t(const CsrDev& d, const CsrKArgs& a, const BwdKArgs& w, cudaStream_t s) {
+  const int64_t nvec = a.N / Tr::kVE;
+  auto go = [&](auto g_tag, auto p_tag) {
+    constexpr int G = decltype(g_tag)::value;
+    constexpr int VPL = decltype(p_tag)::value;
+    const unsigned blocks = (unsigned)((a.n_items * G + kCsrThreads - 1) / kCsrThreads);
+    if (a.N % (G * VPL * Tr::kVE) == 0) csr_backward_vec<Tr, G, VPL, true><<<blocks, kCsrThreads, 0, s>>>(a, w);
+    else csr_backward_vec<Tr, G, VPL, false><<<blocks, kCsrThreads, 0, s>>>(a, w);
+    return cudaGetLastError();
+  };
+  using One = std::integral_constant<int, 1>;
+  using Two = std::integral_constant<int, 2>;
+  cudaError_t e;
+  // two vectors per lane: 16-bit from 16 vectors on, the others where 32 lanes need them
+  if (nvec >= (Tr::kVE == 8 ? 16 : 33)) {
+    switch (next_pow2((nvec + 1) / 2)) {
+      case 8: e = go(std::integral_constant<int, 8>(), Two()); break;
+      case 16: e = go(std::integral_constant<int, 16>(), Two()); break;
+      default: e = go(std::integral_constant<int, 32>(), Two()); break;
+    }
+  } else {
+    switch (next_pow2(nvec)) {
+      case 1: e = go(std::integral_constant<int, 1>(), One()); break;
+      case 2: e = go(std::integral_constant<int, 2>(), One()); break;
+      case 4: e = go(std::integral_constant<int, 4>(), One()); break;
+      case 8: e = go(std::integral_constant<int, 8>(), One()); break;
+      case 16: e = go(std::integral_constant<int, 16>(), One()); break;
+      default: e = go(std::integral_constant<int, 32>(), One()); break;
+    }
+  }
+  return e == cudaSuccess ? launch_split_reduce<Tr>(d, a, s) : e;
+}
+
 }  // namespace
+
+bool csr_backward_applies(const loops_plan_s* p, const void* dC, int64_t lddc, const void* B, int64_t ldb,
+                          const void* dB, int64_t lddb) {
+  const loops_plan_s* t = p->transposed;
+  const int64_t eb = dense_elem_bytes(p->dtype), ec = out_elem_bytes(p->dtype), ve = 16 / eb;
+  if (t->dev.bcsr.n_rb > 0 || t->dev.csr_acc.n_items > 0 || !t->has_vmap || t->vmap.wide ||
+      t->vmap.n_csr != p->nnz)
+    return false;
+  return p->N > 0 && p->N % ve == 0 && p->N / ve <= 64 && (uintptr_t)dC % 16 == 0 && (uintptr_t)B % 16 == 0 &&
+         (uintptr_t)dB % 16 == 0 && (lddc * eb) % 16 == 0 && (ldb * eb) % 16 == 0 && (lddb * ec) % 16 == 0 &&
+         lddc * eb <= (int64_t)UINT32_MAX;
+}
+
+cudaError_t launch_csr_backward(const loops_plan_s* p, const DenseArgs& da, const void* B, int64_t ldb, void* dvals,
+                                const float* b_scale, cudaStream_t s) {
+  const loops_plan_s* t = p->transposed;
+  const CsrDev& d = t->dev.csr;
+  if (d.n_items == 0) return cudaSuccess;
+  const CsrKArgs a = csr_args(p, d, da, false);
+  const BwdKArgs w{B, ldb, dvals, (const int32_t*)t->vmap.csr_src, d.split_row, d.split_slot_ptr, d.n_split,
+                   da.col_scale, b_scale};
+  switch (p->dtype) {
+    case LOOPS_F64: return launch_csr_backward_t<TrF64>(d, a, w, s);
+    case LOOPS_F32: return launch_csr_backward_t<TrF32>(d, a, w, s);
+    case LOOPS_F16: return launch_csr_backward_t<TrF16>(d, a, w, s);
+    case LOOPS_BF16: return launch_csr_backward_t<TrBF16>(d, a, w, s);
+  }
+  return cudaErrorInvalidValue;
+}
 
 cudaError_t launch_csr(const loops_plan_s* p, const CsrDev& d, const DenseArgs& a, bool accumulate,
                        cudaStream_t s) {

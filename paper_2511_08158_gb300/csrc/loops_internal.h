@@ -376,6 +376,13 @@ struct DenseArgs {
 
 cudaError_t launch_csr(const loops_plan_s* p, const CsrDev& d, const DenseArgs& a, bool accumulate,
                        cudaStream_t s);
+// dB and dvals in one pass over the transposed plan: possible when that plan is all CSR (every
+// entry of A is an entry of its CSR items, with 32-bit maps) and rows of dC, B and dB are whole
+// 16-byte vectors, at most 64. `a` describes dB = A^T . dC.
+bool csr_backward_applies(const loops_plan_s* p, const void* dC, int64_t lddc, const void* B, int64_t ldb,
+                          const void* dB, int64_t lddb);
+cudaError_t launch_csr_backward(const loops_plan_s* p, const DenseArgs& a, const void* B, int64_t ldb, void* dvals,
+                                const float* b_scale, cudaStream_t s);
 cudaError_t launch_bcsr(const loops_plan_s* p, const BcsrDev& d, const DenseArgs& a, cudaStream_t s);
 cudaError_t launch_sddmm(const loops_plan_s* p, const void* dC, int64_t lddc, const void* B,
                          int64_t ldb, void* dvals, const float* dc_scale, const float* b_scale, cudaStream_t s);
