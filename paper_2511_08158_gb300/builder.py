@@ -22,6 +22,7 @@ INCLUDE = os.path.join(ROOT, "include")
 SOURCES = ["capi.cpp", "partition.cpp", "layout.cpp", "csr_kernels.cu", "sddmm_kernels.cu", "bcsr_kernels.cu", "csr_noalloc.cu",
            "batched.cu", "batched_plan.cpp", "plan_device.cu", "perf_model.cpp"]
 HEADERS = [os.path.join(CSRC, "loops_internal.h"), os.path.join(CSRC, "device_common.cuh"),
+           os.path.join(CSRC, "value_store.cuh"),
            os.path.join(INCLUDE, "loops.h")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-I", INCLUDE] + ARCH

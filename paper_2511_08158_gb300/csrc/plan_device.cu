@@ -20,6 +20,9 @@
 //      ordered by decreasing length class (stable), values rounded per entry;
 //   6. value maps for loops_plan_set_values, and with want_backward the SDDMM items and the
 //      plan of A^T (a stable sort of the entries by column).
+// With tau = infinity no block can be BCSR: steps 2 to 4 are skipped. 2^18-node graph, 3.6 M
+// entries, FP16: the kernels take 0.18 ms, against 1.8 ms with the sort, a same-address atomic per
+// thread in the validation and one per tile in the block counts.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -27,6 +30,7 @@
 
 #include "device_common.cuh"
 #include "loops_internal.h"
+#include "value_store.cuh"
 
 namespace loops {
 
@@ -298,7 +302,20 @@ __global__ void validate_k(const int64_t* rp, const int32_t* ci, const void* val
       }
     }
   }
-  if (want_max && mx) atomicMax(&st->max_bits, mx);
+  if (want_max) {  // one atomic per block: one per thread on the same word took 0.4 ms
+    __shared__ unsigned long long block_mx[kThreads / 32];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const unsigned long long y = __shfl_xor_sync(0xffffffffu, mx, o);
+      mx = y > mx ? y : mx;
+    }
+    if ((threadIdx.x & 31) == 0) block_mx[threadIdx.x >> 5] = mx;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      for (int w = 1; w < kThreads / 32; ++w) mx = block_mx[w] > mx ? block_mx[w] : mx;
+      if (mx) atomicMax(&st->max_bits, mx);
+    }
+  }
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     st->rp0 = rp[0];
     st->rpn = rp[n_rows];
@@ -306,15 +323,24 @@ __global__ void validate_k(const int64_t* rp, const int32_t* ci, const void* val
 }
 
 // ------------------------------------------------------------------ 2. keys and tiles
-// Row of every entry: the last row i with row_ptr[i] <= k (empty rows are skipped over).
+// Row of every entry: the last row i with row_ptr[i] <= k (empty rows are skipped over). One
+// search per kItems consecutive entries, then forward (searching again past empty rows).
 __global__ void entry_rows_k(const int64_t* rp, int64_t n_rows, int64_t nnz, int32_t* erow) {
-  GS_LOOP(k, nnz) {
-    int64_t lo = 0, hi = n_rows;  // rp[lo] <= k < rp[hi]
-    while (hi - lo > 1) {
-      const int64_t mid = (lo + hi) >> 1;
-      if (rp[mid] <= k) lo = mid; else hi = mid;
+  GS_LOOP(c, (nnz + kItems - 1) / kItems) {
+    int64_t row = -1;
+    const int64_t k1 = min((c + 1) * kItems, nnz);
+    for (int64_t k = c * kItems; k < k1; ++k) {
+      if (row < 0 || rp[row + 1] <= k) {
+        int64_t lo = row < 0 ? 0 : row + 1, hi = n_rows;  // rp[lo] <= k < rp[hi]
+        if (row >= 0 && rp[lo + 1] > k) hi = lo + 1;      // the next row: no search
+        while (hi - lo > 1) {
+          const int64_t mid = (lo + hi) >> 1;
+          if (rp[mid] <= k) lo = mid; else hi = mid;
+        }
+        row = lo;
+      }
+      erow[k] = (int32_t)row;
     }
-    erow[k] = (int32_t)lo;
   }
 }
 
@@ -340,16 +366,28 @@ __global__ void tile_first_k(const int32_t* flag, const int64_t* tpos, int64_t n
   if (blockIdx.x == 0 && threadIdx.x == 0) tile_first[n_t] = nnz;
 }
 
-// Per tile: its block's distinct-column and kept-tile counts, and the first tile of a block.
-__global__ void tile_stats_k(const uint64_t* key, const int64_t* tile_first, int64_t n_t, int cb, int32_t tile_min,
-                             int64_t nb, int32_t* u, int32_t* keep, int64_t* blk_first) {
-  GS_LOOP(t, n_t) {
-    const int64_t b = (int64_t)(key[tile_first[t]] >> cb);
-    BUILD_CHECK(b >= 0 && b < nb);
-    atomicAdd(&u[b], 1);
-    const int64_t cnt = tile_first[t + 1] - tile_first[t];
-    if (tile_min <= 1 || cnt >= tile_min) atomicAdd(&keep[b], 1);
-    if (t == 0 || (int64_t)(key[tile_first[t - 1]] >> cb) != b) blk_first[b] = t;
+// Per row block: its tiles are consecutive (the sort keeps every block's entries in its range of
+// entries), so its first tile and its distinct columns come from the tile numbers at the range's
+// ends; kept tiles are counted by a warp per block where tile_min is on.
+__global__ void block_tiles_k(const int64_t* rp, int64_t n_rows, int64_t nb, int32_t br, const int64_t* tpos,
+                              const int64_t* tile_first, int64_t n_t, int32_t tile_min, int32_t* u, int32_t* keep,
+                              int64_t* blk_first) {
+  const int lane = threadIdx.x & 31;
+  for (int64_t b = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; b < nb;
+       b += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+    const int64_t t0 = tpos[rp[b * br]], t1 = tpos[rp[min((b + 1) * br, n_rows)]];
+    BUILD_CHECK(t0 >= 0 && t0 <= t1 && t1 <= n_t);
+    int32_t kept = (int32_t)(t1 - t0);
+    if (tile_min > 1) {
+      kept = 0;
+      for (int64_t t = t0 + lane; t < t1; t += 32) kept += tile_first[t + 1] - tile_first[t] >= tile_min;
+      kept = (int32_t)__reduce_add_sync(0xffffffffu, (unsigned)kept);
+    }
+    if (lane == 0) {
+      u[b] = (int32_t)(t1 - t0);
+      keep[b] = kept;
+      blk_first[b] = t0;
+    }
   }
 }
 
@@ -599,42 +637,100 @@ __device__ __forceinline__ int bucket_of_len(int64_t len) {  // floor(log2(len +
   return b < 62 ? b : 62;
 }
 
-// Rows of one CSR set: set 0 takes every row of a CSR block (empty rows too), set 1 the rows
-// of BCSR blocks that have moved entries. Rows longer than L become split rows of
-// ceil(len / L) segments.
-__global__ void row_count_k(const int64_t* rp, const uint8_t* is_bcsr, const int32_t* rowlen1, int64_t n_rows,
-                            int32_t br, int which, int64_t L, int64_t* n_items, int64_t* n_slots, int64_t* is_split) {
-  GS_LOOP(i, n_rows) {
-    const bool in_b = is_bcsr[i / br] != 0;
-    int64_t len = -1;
-    if (which == 0 && !in_b) len = rp[i + 1] - rp[i];
-    if (which == 1 && in_b && rowlen1[i] > 0) len = rowlen1[i];
-    const bool sp = len > L;
-    n_items[i] = len < 0 ? 0 : (sp ? (len + L - 1) / L : 1);
-    n_slots[i] = sp ? n_items[i] : 0;
-    is_split[i] = sp ? 1 : 0;
+// Rows of one CSR set: set 0 takes every row of a CSR block (empty rows too; every row when
+// is_bcsr is null), set 1 the rows of BCSR blocks that have moved entries. Rows longer than L
+// become split rows of ceil(len / L) segments.
+struct RowSet {
+  const int64_t* rp;
+  const uint8_t* is_bcsr;
+  const int32_t* rowlen1;
+  int64_t n_rows, L;
+  int32_t br;
+  int which;
+  __device__ __forceinline__ int64_t len(int64_t i) const {  // -1: not in the set
+    const bool in_b = is_bcsr && is_bcsr[i / br] != 0;
+    if (which == 0) return in_b ? -1 : rp[i + 1] - rp[i];
+    return in_b && rowlen1[i] > 0 ? rowlen1[i] : -1;
   }
+};
+
+// Work items, partial-sum slots and split rows, of a row or summed.
+struct RowCount {
+  int64_t items, slots, splits;
+  __device__ __forceinline__ void add(int64_t len, int64_t L) {
+    const int64_t segs = len > L ? (len + L - 1) / L : 0;
+    items += len < 0 ? 0 : (segs ? segs : 1);
+    slots += segs;
+    splits += segs > 0;
+  }
+};
+
+// The items are numbered by one scan of all three counts that recomputes them from the row
+// pointers: sums per tile of kTile rows, their scan (total in sums[blocks]), and the numbers
+// inside a tile where the items are emitted.
+__global__ void __launch_bounds__(kThreads) row_sums_k(RowSet rs, RowCount* sums) {
+  const int64_t base = (int64_t)blockIdx.x * kTile + (int64_t)threadIdx.x * kItems;
+  RowCount c{0, 0, 0}, tot;
+#pragma unroll
+  for (int j = 0; j < kItems; ++j)
+    if (base + j < rs.n_rows) c.add(rs.len(base + j), rs.L);
+  block_excl_scan(c.items, tot.items);
+  block_excl_scan(c.slots, tot.slots);
+  block_excl_scan(c.splits, tot.splits);
+  if (threadIdx.x == 0) sums[blockIdx.x] = tot;
 }
 
-__global__ void row_emit_k(const int64_t* rp, const uint8_t* is_bcsr, const int32_t* rowlen1, const int64_t* cpos,
-                           int64_t n_rows, int32_t br, int which, int64_t L, const int64_t* ibase,
-                           const int64_t* sbase, const int64_t* spidx, int64_t n_slots, int64_t n_split,
-                           int64_t n_items, uint64_t* ikey, int64_t* ival, int32_t* pre_row, int64_t* pre_beg,
-                           int64_t* pre_len, int32_t* split_row, int32_t* split_slot_ptr) {
-  GS_LOOP(i, n_rows) {
-    const bool in_b = is_bcsr[i / br] != 0;
-    int64_t len = -1;
-    if (which == 0 && !in_b) len = rp[i + 1] - rp[i];
-    if (which == 1 && in_b && rowlen1[i] > 0) len = rowlen1[i];
+__global__ void __launch_bounds__(kThreads) row_sums_scan_k(RowCount* sums, int64_t m) {
+  RowCount carry{0, 0, 0};
+  for (int64_t b0 = 0; b0 < m; b0 += kThreads) {
+    const int64_t i = b0 + threadIdx.x;
+    const RowCount v = i < m ? sums[i] : RowCount{0, 0, 0};
+    RowCount tot, at;
+    at.items = carry.items + block_excl_scan(v.items, tot.items);
+    at.slots = carry.slots + block_excl_scan(v.slots, tot.slots);
+    at.splits = carry.splits + block_excl_scan(v.splits, tot.splits);
+    if (i < m) sums[i] = at;
+    carry.items += tot.items;
+    carry.slots += tot.slots;
+    carry.splits += tot.splits;
+  }
+  if (threadIdx.x == 0) sums[m] = carry;
+}
+
+// `total`: the totals of the scan, as read by the host.
+__global__ void __launch_bounds__(kThreads) row_emit_k(RowSet rs, const RowCount* sums, RowCount total,
+                                                       const int64_t* cpos, uint64_t* ikey, int64_t* ival,
+                                                       int32_t* pre_row, int64_t* pre_beg, int64_t* pre_len,
+                                                       int32_t* split_row, int32_t* split_slot_ptr) {
+  const int64_t base = (int64_t)blockIdx.x * kTile + (int64_t)threadIdx.x * kItems;
+  const int64_t L = rs.L;
+  RowCount c{0, 0, 0}, tot;
+  int64_t lens[kItems];
+#pragma unroll
+  for (int j = 0; j < kItems; ++j) {
+    lens[j] = base + j < rs.n_rows ? rs.len(base + j) : -1;
+    c.add(lens[j], L);
+  }
+  RowCount at = sums[blockIdx.x];
+  at.items += block_excl_scan(c.items, tot.items);
+  at.slots += block_excl_scan(c.slots, tot.slots);
+  at.splits += block_excl_scan(c.splits, tot.splits);
+#pragma unroll
+  for (int j = 0; j < kItems; ++j) {
+    const int64_t i = base + j, len = lens[j];
     if (len < 0) continue;
-    const int64_t beg = cpos[rp[i]];  // canonical position of the row's first entry in this set
-    int64_t it = ibase[i];
-    BUILD_CHECK(it >= 0 && it + (len > L ? (len + L - 1) / L : 1) <= n_items);
+    RowCount next = at;
+    next.add(len, L);
+    const int64_t it0 = at.items, slot0 = at.slots, sp = at.splits;
+    at = next;
+    BUILD_CHECK(it0 >= 0 && next.items <= total.items);
+    // canonical position of the row's first entry in this set (its own entries where all are)
+    const int64_t beg = cpos ? cpos[rs.rp[i]] : rs.rp[i];
     if (len > L) {
-      int64_t slot = sbase[i];
-      BUILD_CHECK(split_row && spidx[i] >= 0 && spidx[i] < n_split);
-      split_row[spidx[i]] = (int32_t)i;
-      split_slot_ptr[spidx[i]] = (int32_t)slot;
+      BUILD_CHECK(split_row && sp >= 0 && sp < total.splits);
+      split_row[sp] = (int32_t)i;
+      split_slot_ptr[sp] = (int32_t)slot0;
+      int64_t it = it0, slot = slot0;
       for (int64_t s0 = 0; s0 < len; s0 += L, ++it, ++slot) {
         pre_row[it] = (int32_t)(-1 - slot);
         pre_beg[it] = beg + s0;
@@ -643,14 +739,14 @@ __global__ void row_emit_k(const int64_t* rp, const uint8_t* is_bcsr, const int3
         ival[it] = it;
       }
     } else {
-      pre_row[it] = (int32_t)i;
-      pre_beg[it] = beg;
-      pre_len[it] = len;
-      ikey[it] = LOOPS_CSR_ITEMS_BY_LENGTH ? (uint64_t)(63 - bucket_of_len(len)) : 0;
-      ival[it] = it;
+      pre_row[it0] = (int32_t)i;
+      pre_beg[it0] = beg;
+      pre_len[it0] = len;
+      ikey[it0] = LOOPS_CSR_ITEMS_BY_LENGTH ? (uint64_t)(63 - bucket_of_len(len)) : 0;
+      ival[it0] = it0;
     }
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0 && split_slot_ptr) split_slot_ptr[n_split] = (int32_t)n_slots;
+  if (blockIdx.x == 0 && threadIdx.x == 0 && split_slot_ptr) split_slot_ptr[total.splits] = (int32_t)total.slots;
 }
 
 __global__ void item_order_k(const int64_t* order, int64_t n, const int32_t* pre_row, const int64_t* pre_len,
@@ -663,32 +759,55 @@ __global__ void item_order_k(const int64_t* order, int64_t n, const int32_t* pre
   }
 }
 
-// One warp per item: columns and rounded values of its entries, and the value map.
-template <class TB>
-__global__ void item_gather_k(const int64_t* order, int64_t n, const int64_t* pre_beg, const int64_t* item_ptr,
-                              const int64_t* canon_src, int64_t n_canon, int64_t total, const int32_t* ci,
-                              const void* vals, int vf32, double scale, double tiny, const int64_t* remap,
-                              int32_t* col, TB* val, int64_t* csr_src, unsigned long long* n_sub) {
-  const int lane = threadIdx.x & 31;
-  for (int64_t q = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; q < n;
-       q += ((int64_t)gridDim.x * blockDim.x) >> 5) {
-    const int64_t b = pre_beg[order[q]];
-    const int64_t d0 = item_ptr[q], len = item_ptr[q + 1] - d0;
-    BUILD_CHECK(b >= 0 && b + len <= n_canon && d0 >= 0 && d0 + len <= total);
-    unsigned long long sub = 0;
-    for (int64_t e = lane; e < len; e += 32) {
-      const int64_t k = canon_src[b + e];
-      col[d0 + e] = ci[k];
-      const TB x = from_f64<TB>(load_val(vals, vf32, k) * scale);
-      val[d0 + e] = x;
-      if (csr_src) csr_src[d0 + e] = remap ? remap[k] : k;
-      if (tiny > 0.0) {
-        const double y = (double)(float)x;
-        sub += (y != 0.0 && fabs(y) < tiny);
+// G lanes per item: columns and rounded values of its entries, and the value map (32-bit indices,
+// or 64-bit when wide). canon_src null: canonical positions are input entries.
+struct ItemGatherArgs {
+  const int64_t* order;
+  int64_t n;
+  const int64_t* pre_beg;
+  const int64_t* item_ptr;
+  const int64_t* canon_src;
+  int64_t n_canon, total;
+  const int32_t* ci;
+  const void* vals;
+  double scale;
+  float scale_f;
+  float tiny;                // smallest normal of a 16-bit dtype (0 otherwise)
+  const int64_t* remap;
+  int32_t* col;
+  void* val;
+  void* csr_src;             // may be null
+  int wide;
+  unsigned long long* n_sub;
+};
+
+template <class TB, class TIn, int G>
+__global__ void __launch_bounds__(kThreads) item_gather_k(ItemGatherArgs a) {
+  const int sub = threadIdx.x & (G - 1);
+  const TIn* vals = reinterpret_cast<const TIn*>(a.vals);
+  unsigned long long n_sub = 0;
+  for (int64_t q = ((int64_t)blockIdx.x * kThreads + threadIdx.x) / G; q < a.n;
+       q += (int64_t)gridDim.x * (kThreads / G)) {
+    const int64_t b = a.pre_beg[a.order[q]];
+    const int64_t d0 = a.item_ptr[q], len = a.item_ptr[q + 1] - d0;
+    BUILD_CHECK(b >= 0 && b + len <= a.n_canon && d0 >= 0 && d0 + len <= a.total);
+    for (int64_t e = sub; e < len; e += G) {
+      const int64_t k = a.canon_src ? a.canon_src[b + e] : b + e;
+      a.col[d0 + e] = a.ci[k];
+      const TB x = stored_value<TB>(vals[k], a.scale, a.scale_f);
+      reinterpret_cast<TB*>(a.val)[d0 + e] = x;
+      if (a.csr_src) {
+        const int64_t src = a.remap ? a.remap[k] : k;
+        if (a.wide) reinterpret_cast<int64_t*>(a.csr_src)[d0 + e] = src;
+        else reinterpret_cast<int32_t*>(a.csr_src)[d0 + e] = (int32_t)src;
+      }
+      if constexpr (sizeof(TB) == 2) {
+        const float y = fabsf((float)x);
+        n_sub += y != 0.f && y < a.tiny;
       }
     }
-    if (sub) atomicAdd(n_sub, sub);
   }
+  if (n_sub) atomicAdd(a.n_sub, n_sub);
 }
 
 __global__ void narrow_k(const int64_t* in, int64_t n, int32_t* out) {
@@ -771,15 +890,14 @@ cudaError_t launch_tile_values(const TileArgs& a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-template <class TB>
-cudaError_t launch_item_gather(const int64_t* order, int64_t n, const int64_t* pre_beg, const int64_t* item_ptr,
-                               const int64_t* canon_src, int64_t n_canon, int64_t total, const DevCsrIn& A,
-                               double scale, double tiny, const int64_t* remap, int32_t* col, void* val,
-                               int64_t* csr_src, unsigned long long* n_sub, cudaStream_t s) {
-  const unsigned blocks = (unsigned)std::max<int64_t>(1, std::min<int64_t>((n * 32 + kThreads - 1) / kThreads, 152 * 16));
-  item_gather_k<TB><<<blocks, kThreads, 0, s>>>(order, n, pre_beg, item_ptr, canon_src, n_canon, total, A.ci,
-                                                 A.vals, A.vals_f32, scale, tiny, remap, col, (TB*)val, csr_src,
-                                                 n_sub);
+// 8 lanes per item for short items (four items per warp), a warp for long ones
+template <class TB, class TIn>
+cudaError_t launch_item_gather(const ItemGatherArgs& a, cudaStream_t s) {
+  const bool narrow = a.total < 24 * a.n;
+  const int64_t lanes = a.n * (narrow ? 8 : 32);
+  const unsigned blocks = (unsigned)std::max<int64_t>(1, std::min<int64_t>((lanes + kThreads - 1) / kThreads, 152 * 16));
+  if (narrow) item_gather_k<TB, TIn, 8><<<blocks, kThreads, 0, s>>>(a);
+  else item_gather_k<TB, TIn, 32><<<blocks, kThreads, 0, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -793,20 +911,17 @@ cudaError_t dispatch_tile_values(loops_dtype d, const TileArgs& a, cudaStream_t 
   return cudaErrorInvalidValue;
 }
 
-cudaError_t dispatch_item_gather(loops_dtype d, const int64_t* order, int64_t n, const int64_t* pre_beg,
-                                 const int64_t* item_ptr, const int64_t* canon_src, int64_t n_canon, int64_t total,
-                                 const DevCsrIn& A, double scale, double tiny, const int64_t* remap, int32_t* col,
-                                 void* val, int64_t* csr_src, unsigned long long* n_sub, cudaStream_t s) {
-#define LOOPS_GATHER(TB) \
-  launch_item_gather<TB>(order, n, pre_beg, item_ptr, canon_src, n_canon, total, A, scale, tiny, remap, col, val, \
-                         csr_src, n_sub, s)
+cudaError_t dispatch_item_gather(loops_dtype d, int vals_f32, const ItemGatherArgs& a, cudaStream_t s) {
   switch (d) {
-    case LOOPS_F64: return LOOPS_GATHER(double);
-    case LOOPS_F32: return LOOPS_GATHER(float);
-    case LOOPS_F16: return LOOPS_GATHER(__half);
-    case LOOPS_BF16: return LOOPS_GATHER(__nv_bfloat16);
+    case LOOPS_F64:
+      return vals_f32 ? launch_item_gather<double, float>(a, s) : launch_item_gather<double, double>(a, s);
+    case LOOPS_F32:
+      return vals_f32 ? launch_item_gather<float, float>(a, s) : launch_item_gather<float, double>(a, s);
+    case LOOPS_F16:
+      return vals_f32 ? launch_item_gather<__half, float>(a, s) : launch_item_gather<__half, double>(a, s);
+    case LOOPS_BF16:
+      return vals_f32 ? launch_item_gather<__nv_bfloat16, float>(a, s) : launch_item_gather<__nv_bfloat16, double>(a, s);
   }
-#undef LOOPS_GATHER
   return cudaErrorInvalidValue;
 }
 
@@ -815,48 +930,49 @@ cudaError_t reset_build_err(cudaStream_t s) {
   return cudaMemcpyToSymbolAsync(g_build_err, &zero, sizeof(int), 0, cudaMemcpyHostToDevice, s);
 }
 
+loops_status build_err_status(bool failed, const char* what) {
+  if (!failed) return LOOPS_OK;
+  set_error(std::string(what) + ": an index check failed (access skipped); the plan was not built");
+  return LOOPS_ERR_STATE;
+}
+
 // After a build stage: a recorded index check fails the build (no access was made).
 loops_status check_build_err(cudaStream_t s, const char* what) {
   int h = 0;
   cudaError_t e = cudaMemcpyFromSymbolAsync(&h, g_build_err, sizeof(int), 0, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_status(e, what);
-  if (h) {
-    set_error(std::string(what) + ": an index check failed (access skipped); the plan was not built");
-    return LOOPS_ERR_STATE;
-  }
-  return LOOPS_OK;
+  return build_err_status(h != 0, what);
 }
 
 #define TRY(x) do { cudaError_t e_ = (x); if (e_ != cudaSuccess) return cuda_status(e_, what); } while (0)
 #define NEED(ptr) do { if (!(ptr)) return cuda_status(ar.err, what); } while (0)
 
-// One CSR set (0: rows of CSR blocks, 1: moved entries of BCSR blocks) into its work items.
-loops_status build_csr_set(loops_plan_s* p, const DevCsrIn& A, const int64_t* remap, int which, const uint8_t* cls,
-                           const uint8_t* is_bcsr, const int32_t* rowlen1, const int64_t* cpos, const int64_t* csrc,
-                           int64_t n_canon, int64_t N, double tiny, unsigned long long* n_sub, int64_t** csr_src_out, int64_t* n_src,
-                           Arena& ar, cudaStream_t s) {
+// One CSR set (0: rows of CSR blocks, 1: moved entries of BCSR blocks) into its work items. cpos
+// (canonical position of every entry) and csrc (its inverse) are null where every entry is in
+// the set. With `csr_src` the plan gets the set's value map (*csr_src, n_canon entries).
+loops_status build_csr_set(loops_plan_s* p, const DevCsrIn& A, const int64_t* remap, int which, const uint8_t* is_bcsr,
+                           const int32_t* rowlen1, const int64_t* cpos, const int64_t* csrc, int64_t n_canon,
+                           int64_t N, double tiny, unsigned long long* n_sub, void** csr_src, bool wide, Arena& ar,
+                           cudaStream_t s) {
   const char* what = "device plan build (CSR part)";
   CsrDev& cd = which == 0 ? p->dev.csr : p->dev.csr_acc;
   int64_t& bytes = p->dev.device_bytes;
-  const int64_t n = A.n_rows, L = std::max<int64_t>(p->split_len, 1);
-  int64_t* n_items_r = ar.get<int64_t>(n + 1);
-  int64_t* n_slots_r = ar.get<int64_t>(n + 1);
-  int64_t* split_r = ar.get<int64_t>(n + 1);
-  NEED(split_r);
-  if (n) row_count_k<<<grid_for(n), kThreads, 0, s>>>(A.rp, is_bcsr, rowlen1, n, p->br, which, L, n_items_r,
-                                                      n_slots_r, split_r);
+  const int64_t n = A.n_rows;
+  if (n == 0) return LOOPS_OK;
+  const RowSet rs{A.rp, is_bcsr, rowlen1, n, std::max<int64_t>(p->split_len, 1), p->br, which};
+  const int64_t row_blocks = (n + kTile - 1) / kTile;
+  RowCount* sums = ar.get<RowCount>(row_blocks + 1);
+  NEED(sums);
+  row_sums_k<<<(unsigned)row_blocks, kThreads, 0, s>>>(rs, sums);
+  row_sums_scan_k<<<1, kThreads, 0, s>>>(sums, row_blocks);
   TRY(cudaGetLastError());
-  TRY(excl_scan<int64_t>(n_items_r, n_items_r, n, true, ar, s));
-  TRY(excl_scan<int64_t>(n_slots_r, n_slots_r, n, true, ar, s));
-  TRY(excl_scan<int64_t>(split_r, split_r, n, true, ar, s));
-  int64_t n_it = 0, n_sl = 0, n_sp = 0;
-  TRY(to_host(&n_it, n_items_r + n, s));
-  TRY(to_host(&n_sl, n_slots_r + n, s));
-  TRY(to_host(&n_sp, split_r + n, s));
+  RowCount total{0, 0, 0};
+  TRY(to_host(&total, sums + row_blocks, s));
+  const int64_t n_it = total.items;
   cd.n_items = n_it;
-  cd.n_slots = n_sl;
-  cd.n_split = n_sp;
+  cd.n_slots = total.slots;
+  cd.n_split = total.splits;
   if (n_it == 0) return LOOPS_OK;
   uint64_t* ikey = ar.get<uint64_t>(n_it);
   uint64_t* ikey2 = ar.get<uint64_t>(n_it);
@@ -867,13 +983,12 @@ loops_status build_csr_set(loops_plan_s* p, const DevCsrIn& A, const int64_t* re
   int64_t* pre_len = ar.get<int64_t>(n_it);
   int64_t* dlen = ar.get<int64_t>(n_it + 1);
   NEED(dlen);
-  if (n_sp) {
-    TRY(own(&cd.split_row, n_sp, bytes));
-    TRY(own(&cd.split_slot_ptr, n_sp + 1, bytes));
+  if (total.splits) {
+    TRY(own(&cd.split_row, total.splits, bytes));
+    TRY(own(&cd.split_slot_ptr, total.splits + 1, bytes));
   }
-  row_emit_k<<<grid_for(n), kThreads, 0, s>>>(A.rp, is_bcsr, rowlen1, cpos, n, p->br, which, L, n_items_r, n_slots_r,
-                                              split_r, n_sl, n_sp, n_it, ikey, ival, pre_row, pre_beg, pre_len,
-                                              cd.split_row, cd.split_slot_ptr);
+  row_emit_k<<<(unsigned)row_blocks, kThreads, 0, s>>>(rs, sums, total, cpos, ikey, ival, pre_row, pre_beg, pre_len,
+                                                       cd.split_row, cd.split_slot_ptr);
   TRY(cudaGetLastError());
   TRY(radix_sort<int64_t>(&ikey, &ival, &ikey2, &ival2, n_it, 6, ar, s));
   TRY(own(&cd.item_row, n_it, bytes));
@@ -881,27 +996,21 @@ loops_status build_csr_set(loops_plan_s* p, const DevCsrIn& A, const int64_t* re
   item_order_k<<<grid_for(n_it), kThreads, 0, s>>>(ival, n_it, pre_row, pre_len, cd.item_row, dlen);
   TRY(cudaGetLastError());
   TRY(excl_scan<int64_t>(dlen, cd.item_ptr, n_it, true, ar, s));
-  int64_t total = 0;
-  TRY(to_host(&total, cd.item_ptr + n_it, s));
-  cd.nnz = total;
+  cd.nnz = n_canon;  // the set's rows hold exactly its entries
   const int es = dense_elem_bytes(p->dtype);
-  TRY(own(&cd.col, total, bytes));
-  TRY(own((uint8_t**)&cd.val, total * es, bytes));
-  int64_t* csr_src = nullptr;
-  if (csr_src_out) {
-    csr_src = ar.get<int64_t>(total);
-    NEED(csr_src);
+  TRY(own(&cd.col, n_canon, bytes));
+  TRY(own((uint8_t**)&cd.val, n_canon * es, bytes));
+  if (csr_src && wide) TRY(own((int64_t**)csr_src, n_canon, p->vmap.bytes));
+  if (csr_src && !wide) TRY(own((int32_t**)csr_src, n_canon, p->vmap.bytes));
+  if (n_canon) {
+    const ItemGatherArgs ga{ival, n_it, pre_beg, cd.item_ptr, csrc, n_canon, n_canon, A.ci, A.vals, p->scale,
+                            scale_f32(p->scale), (float)tiny, remap, cd.col, cd.val, csr_src ? *csr_src : nullptr,
+                            wide ? 1 : 0, n_sub};
+    TRY(dispatch_item_gather(p->dtype, A.vals_f32, ga, s));
   }
-  if (total)
-    TRY(dispatch_item_gather(p->dtype, ival, n_it, pre_beg, cd.item_ptr, csrc, n_canon, total, A, p->scale, tiny,
-                             remap, cd.col, cd.val, csr_src, n_sub, s));
-  if (n_sl) {
+  if (total.slots) {
     const int acc_bytes = p->dtype == LOOPS_F64 ? 8 : 4;
-    TRY(own((uint8_t**)&cd.scratch, n_sl * std::max<int64_t>(N, 1) * acc_bytes, bytes));
-  }
-  if (csr_src_out) {
-    *csr_src_out = csr_src;
-    *n_src = total;
+    TRY(own((uint8_t**)&cd.scratch, total.slots * std::max<int64_t>(N, 1) * acc_bytes, bytes));
   }
   return LOOPS_OK;
 }
@@ -980,10 +1089,37 @@ loops_status build_part_device(loops_plan_s* p, const DevCsrIn& A, const int64_t
   const int bb = bit_width(nb > 1 ? (uint64_t)(nb - 1) : 1);
   const int32_t tile_min = p->tile_min;
   const double tiny = p->dtype == LOOPS_F16 ? std::ldexp(1.0, -14) : p->dtype == LOOPS_BF16 ? std::ldexp(1.0, -126) : 0.0;
-  unsigned long long* n_sub = ar.get<unsigned long long>(1);
+  unsigned long long* n_sub = ar.get<unsigned long long>(2);  // [1]: the build's error word, for one read of both
   NEED(n_sub);
-  TRY(cudaMemsetAsync(n_sub, 0, sizeof(unsigned long long), s));
+  TRY(cudaMemsetAsync(n_sub, 0, 2 * sizeof(unsigned long long), s));
   TRY(reset_build_err(s));
+  auto finish = [&]() -> loops_status {
+    unsigned long long h[2] = {0, 0};
+    TRY(cudaMemcpyFromSymbolAsync(n_sub + 1, g_build_err, sizeof(int), 0, cudaMemcpyDeviceToDevice, s));
+    TRY(cudaMemcpyAsync(h, n_sub, sizeof(h), cudaMemcpyDeviceToHost, s));
+    TRY(cudaStreamSynchronize(s));
+    p->n_subnormal = (int64_t)h[0];
+    return build_err_status(h[1] != 0, what);
+  };
+
+  // tau = infinity: no block reaches it, so every row is in the CSR part and its entries keep
+  // their input order; nothing is sorted or counted per block
+  if (!contiguous && std::isinf(tau)) {
+    p->n_csr_rows = n;
+    p->nnz_csr = nnz;
+    p->nnz_bcsr = p->n_rb = p->n_tiles = 0;
+    ValueMapDev& m = p->vmap;
+    if (want_maps) {
+      free_value_maps(m);
+      m.n_csr = nnz;
+      m.wide = value_maps_wide(nnz, 0);
+    }
+    const loops_status st = build_csr_set(p, A, remap, 0, nullptr, nullptr, nullptr, nullptr, nnz, N, tiny, n_sub,
+                                          want_maps ? &m.csr_src : nullptr, m.wide, ar, s);
+    if (st) return st;
+    p->has_vmap = want_maps;
+    return finish();
+  }
 
   // ---- 2. entries sorted by (row block, column), ties in input order; tiles are the runs
   int32_t* erow = ar.get<int32_t>(nnz);
@@ -1004,13 +1140,15 @@ loops_status build_part_device(loops_plan_s* p, const DevCsrIn& A, const int64_t
   uint8_t* cls = ar.get<uint8_t>(nnz);
   int32_t* rowlen1 = ar.get<int32_t>(n);
   NEED(rowlen1);
-  TRY(cudaMemsetAsync(u, 0, (size_t)std::max<int64_t>(nb, 1) * 4, s));
-  TRY(cudaMemsetAsync(keep, 0, (size_t)std::max<int64_t>(nb, 1) * 4, s));
+  if (!nnz) {  // otherwise block_tiles_k writes them
+    TRY(cudaMemsetAsync(u, 0, (size_t)std::max<int64_t>(nb, 1) * 4, s));
+    TRY(cudaMemsetAsync(keep, 0, (size_t)std::max<int64_t>(nb, 1) * 4, s));
+  }
   TRY(cudaMemsetAsync(rowlen1, 0, (size_t)std::max<int64_t>(n, 1) * 4, s));
   int64_t n_t = 0;
   int64_t* tile_first = nullptr;
   if (nnz) {
-    entry_rows_k<<<grid_for(nnz), kThreads, 0, s>>>(A.rp, n, nnz, erow);
+    entry_rows_k<<<grid_for((nnz + kItems - 1) / kItems), kThreads, 0, s>>>(A.rp, n, nnz, erow);
     make_keys_k<<<grid_for(nnz), kThreads, 0, s>>>(A.ci, erow, nnz, br, cb, key, idx);
     TRY(cudaGetLastError());
     TRY(radix_sort<int64_t>(&key, &idx, &key2, &idx2, nnz, cb + bb, ar, s));
@@ -1021,7 +1159,8 @@ loops_status build_part_device(loops_plan_s* p, const DevCsrIn& A, const int64_t
     tile_first = ar.get<int64_t>(n_t + 1);
     NEED(tile_first);
     tile_first_k<<<grid_for(nnz), kThreads, 0, s>>>(flag, tpos, nnz, tile_first, n_t);
-    tile_stats_k<<<grid_for(n_t), kThreads, 0, s>>>(key, tile_first, n_t, cb, tile_min, nb, u, keep, blk_first);
+    block_tiles_k<<<grid_for(nb * 32), kThreads, 0, s>>>(A.rp, n, nb, br, tpos, tile_first, n_t, tile_min, u, keep,
+                                                         blk_first);
     TRY(cudaGetLastError());
   }
 
@@ -1056,6 +1195,7 @@ loops_status build_part_device(loops_plan_s* p, const DevCsrIn& A, const int64_t
   // ---- 4. BCSR part
   int64_t* slot_ptr = nullptr;
   int64_t* slot_src = nullptr;
+  int64_t n_slot_src = 0;
   const int64_t n_fslots = n_tiles * br;
   if (n_rb) {
     const int es = dense_elem_bytes(p->dtype);
@@ -1104,13 +1244,12 @@ loops_status build_part_device(loops_plan_s* p, const DevCsrIn& A, const int64_t
     TRY(dispatch_tile_values(p->dtype, ta, s));
     if (want_maps) {
       TRY(excl_scan<int64_t>(slot_cnt, slot_ptr, n_fslots, true, ar, s));
-      int64_t n_src = 0;
-      TRY(to_host(&n_src, slot_ptr + n_fslots, s));
-      slot_src = ar.get<int64_t>(n_src);
+      TRY(to_host(&n_slot_src, slot_ptr + n_fslots, s));
+      slot_src = ar.get<int64_t>(n_slot_src);
       NEED(slot_src);
       ta.slot_ptr = slot_ptr;
       ta.slot_src = slot_src;
-      ta.n_src = n_src;
+      ta.n_src = n_slot_src;
       tile_srcmap_k<<<grid_for(n_t), kThreads, 0, s>>>(ta);
       TRY(cudaGetLastError());
     }
@@ -1184,14 +1323,18 @@ loops_status build_part_device(loops_plan_s* p, const DevCsrIn& A, const int64_t
     canon_src_k<<<grid_for(nnz), kThreads, 0, s>>>(cls, c1, nnz, 1, nnz1, src1);
     TRY(cudaGetLastError());
   }
-  int64_t* csr_src = nullptr;
-  int64_t n_csr_src = 0;
+  ValueMapDev& m = p->vmap;
+  if (want_maps) {
+    free_value_maps(m);
+    m.n_csr = nnz0;
+    m.n_slots = n_fslots;
+    m.wide = value_maps_wide(nnz, n_fslots);
+  }
   loops_status st;
-  if ((st = build_csr_set(p, A, remap, 0, cls, is_bcsr, rowlen1, c0, src0, nnz0, N, tiny, n_sub,
-                          want_maps ? &csr_src : nullptr, &n_csr_src, ar, s)))
+  if ((st = build_csr_set(p, A, remap, 0, is_bcsr, rowlen1, c0, src0, nnz0, N, tiny, n_sub,
+                          want_maps ? &m.csr_src : nullptr, m.wide, ar, s)))
     return st;
-  if ((st = build_csr_set(p, A, remap, 1, cls, is_bcsr, rowlen1, c1, src1, nnz1, N, tiny, n_sub, nullptr, nullptr,
-                          ar, s)))
+  if ((st = build_csr_set(p, A, remap, 1, is_bcsr, rowlen1, c1, src1, nnz1, N, tiny, n_sub, nullptr, false, ar, s)))
     return st;
   // canonical CSR rows: every row of a CSR block, plus the rows with moved entries. Row blocks
   // hold B_r rows except possibly the last one.
@@ -1206,13 +1349,8 @@ loops_status build_part_device(loops_plan_s* p, const DevCsrIn& A, const int64_t
   p->nnz_csr = nnz0 + nnz1;
   p->nnz_bcsr = nnz - nnz0 - nnz1;
 
-  // ---- 6. value maps
+  // ---- 6. value maps of the BCSR part
   if (want_maps) {
-    ValueMapDev& m = p->vmap;
-    free_value_maps(m);
-    m.n_csr = n_csr_src;
-    m.n_slots = n_fslots;
-    m.wide = value_maps_wide(nnz, n_fslots);
     // owned copies, narrowed to 32 bits where they fit
     auto keep_map = [&](void** dst, const int64_t* src, int64_t count) -> cudaError_t {
       if (count <= 0) return cudaSuccess;
@@ -1225,19 +1363,13 @@ loops_status build_part_device(loops_plan_s* p, const DevCsrIn& A, const int64_t
       narrow_k<<<grid_for(count), kThreads, 0, s>>>(src, count, (int32_t*)*dst);
       return cudaGetLastError();
     };
-    TRY(keep_map(&m.csr_src, csr_src, n_csr_src));
     if (n_fslots) {
-      int64_t n_src = 0;
-      TRY(to_host(&n_src, slot_ptr + n_fslots, s));
       TRY(keep_map(&m.bcsr_ptr, slot_ptr, n_fslots + 1));
-      TRY(keep_map(&m.bcsr_src, slot_src, n_src));
+      TRY(keep_map(&m.bcsr_src, slot_src, n_slot_src));
     }
     p->has_vmap = true;
   }
-  unsigned long long sub = 0;
-  TRY(to_host(&sub, n_sub, s));
-  p->n_subnormal = (int64_t)sub;
-  return check_build_err(s, what);
+  return finish();
 }
 
 // SDDMM items of A's own pattern (rows cut at L entries, stably ordered by decreasing length)

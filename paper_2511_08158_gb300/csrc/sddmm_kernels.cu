@@ -7,6 +7,7 @@
 
 #include "device_common.cuh"
 #include "loops_internal.h"
+#include "value_store.cuh"
 
 // SDDMM: reduce the four in-flight entries' partial dot products with one butterfly (1) or each
 // with its own shuffle tree (0).
@@ -295,13 +296,6 @@ __global__ void colscale_kernel(float* __restrict__ s, int64_t cols) {
   s[c] = r;
 }
 
-template <class T>
-__device__ __forceinline__ T cvt_rn(float x);
-template <>
-__device__ __forceinline__ __half cvt_rn<__half>(float x) { return __float2half_rn(x); }
-template <>
-__device__ __forceinline__ __nv_bfloat16 cvt_rn<__nv_bfloat16>(float x) { return __float2bfloat16_rn(x); }
-
 // The scales are powers of two: x / s equals x * (1 / s) bit for bit wherever 1 / s is a
 // binary32 number (s >= 2^-127); smaller scales divide.
 __device__ __forceinline__ float unscale(float x, float s, float inv, bool mul) { return mul ? x * inv : x / s; }
@@ -357,28 +351,6 @@ __global__ void __launch_bounds__(kCastThreads) scale_cast_kernel(const float* _
 
 // ------------------------------------------------------------------ value refresh from device
 
-// Out of line: inlined, the compiler computes it for every entry and selects.
-template <class TB>
-__device__ __noinline__ TB stored_value_f64(float v, double scale) { return from_f64<TB>((double)v * scale); }
-
-// Stored value of one input entry: round(scale * v). A binary32 entry's product with the power-of-
-// two scale is exact in binary32, so it needs no binary64 arithmetic (a slow pipe here), except
-// below binary32's normal range.
-template <class TB>
-__device__ __forceinline__ TB stored_value(double v, double scale, float) { return from_f64<TB>(v * scale); }
-template <class TB>
-__device__ __forceinline__ TB stored_value(float v, double scale, float scale_f) {
-  if constexpr (std::is_same<TB, double>::value) {
-    return (double)v * scale;
-  } else if constexpr (std::is_same<TB, float>::value) {
-    return v;  // FP32 plans store unscaled values
-  } else {
-    const float x = v * scale_f;  // scale_f 0: the scale is outside binary32's normal range
-    if (v != 0.f && !(fabsf(x) >= 0x1p-126f)) return stored_value_f64<TB>(v, scale);
-    return cvt_rn<TB>(x);
-  }
-}
-
 // Stored value = round(scale * sum of the slot's input entries in input order), as the host
 // packer does: CSR positions have one source each, BCSR fragment slots zero or more. Bound by
 // the gathers of `vals` through the map: kSetU positions per thread are in flight, a block's
@@ -420,9 +392,8 @@ cudaError_t launch_set_values_i(const loops_plan_s* p, const TIn* vals, cudaStre
   // kSetU positions per thread until the grid fills the chip (8 blocks of 256 per SM)
   const int64_t need = std::max((m.n_csr + kSetU - 1) / kSetU, m.n_slots);
   const unsigned blocks = (unsigned)std::max<int64_t>(1, std::min<int64_t>((need + 255) / 256, 152 * 8));
-  const float scale_f = p->scale >= 0x1p-126 && p->scale <= 0x1p127 ? (float)p->scale : 0.f;
   set_values_kernel<TB, TIn, TIdx><<<blocks, 256, 0, s>>>(
-      vals, p->scale, scale_f, (const TIdx*)m.csr_src, m.n_csr, (TB*)p->dev.csr.val, (const TIdx*)m.bcsr_ptr,
+      vals, p->scale, scale_f32(p->scale), (const TIdx*)m.csr_src, m.n_csr, (TB*)p->dev.csr.val, (const TIdx*)m.bcsr_ptr,
       (const TIdx*)m.bcsr_src, m.n_slots, (TB*)p->dev.bcsr.tile_val);
   return cudaGetLastError();
 }
