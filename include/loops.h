@@ -6,7 +6,7 @@
  * vector-wise BCSR part of B_r x 1 tiles (the LOOPS format, Sec. 3.2.1; conversion,
  * Algorithm 1), and the SpMM runs both parts on one GPU: the CSR part on CUDA cores (the
  * AXPY row kernel of Sec. 3.3), the BCSR part on tensor cores (the outer-product tile kernel,
- * Algorithms 2 and 3) -- FP64 DMMA, FP16/BF16 MMA with FP32 accumulation -- or, for FP32, on a
+ * Algorithms 2 and 3) -- FP16/BF16 MMA with FP32 accumulation -- or, for FP64 and FP32, on a
  * register-blocked CUDA-core outer product. Each output row has exactly one writer, so the
  * result is deterministic and needs no atomics (Sec. 3.4).
  *
@@ -20,7 +20,7 @@
  *    not synchronise the device unless its comment says so.
  *  - Element types per plan dtype:
  *        dtype      A values stored   B, dC      C, dB, dvals   accumulation
- *        LOOPS_F64  f64               f64        f64            f64 (DFMA / DMMA)
+ *        LOOPS_F64  f64               f64        f64            f64 (DFMA)
  *        LOOPS_F32  f32               f32        f32            f32 (FFMA)
  *        LOOPS_F16  f16 (x s_A)       f16        f32            f32 (HMMA)
  *        LOOPS_BF16 bf16 (x s_A)      bf16       f32            f32 (HMMA)

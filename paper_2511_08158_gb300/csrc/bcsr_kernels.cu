@@ -1,4 +1,4 @@
-// BCSR-part SpMM: the outer-product tile kernel of Algorithms 2 and 3, on tensor cores.
+// BCSR-part SpMM: the outer-product tile kernel of Algorithms 2 and 3; 16-bit tiles on tensor cores.
 //
 // A row block of B_r rows holds tiles (B_r x 1 columns of A, one per distinct column) padded
 // to a multiple of the MMA K. Kernels run over work units (a block, or a K-aligned range of a
@@ -11,8 +11,8 @@
 //             The 16 B rows of a group are staged in shared memory by bulk copies of the
 //             TMA engine (cp.async.bulk + mbarrier, a ring of stages) and transposed into B
 //             fragments with ldmatrix.trans; padded tiles (col -1) are zero rows.
-//   F64       mma.sync m8n8k4 (DMMA). A lane's B fragment is one element, so B is read
-//             straight from global memory with 16-byte loads, two N-fragments per load.
+//   F64       FP64 FMAs on the entries of each group of 4 tiles (the FP64 MMA runs on the same
+//             pipe, slower, and multiplies the tiles' zeros).
 //   F32       CUDA-core register-blocked outer product (TF32 MMA would not meet FP32
 //             accuracy): a group of lanes owns B_r x 4*G outputs and updates them per tile.
 #include "device_common.cuh"
@@ -254,18 +254,21 @@ cudaError_t launch_hmma(const BcsrKArgs& a, int ntile, cudaStream_t s) {
   return launch_hmma_cfg<T, 4, 4>(a, bulk, s);
 }
 
-// ------------------------------------------------------------------ F64: m8n8k4 DMMA
-__device__ __forceinline__ void dmma884(double (&d)[2], double a, double b) {
-  asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0,%1}, {%2}, {%3}, {%0,%1};"
-               : "+d"(d[0]), "+d"(d[1]) : "d"(a), "d"(b));
-}
-
-// One warp per (row block, 16*NP columns). Lane (q, t) = (lane / 4, lane % 4) holds A[q][t] of
-// the group and loads B[col_t][n0 + 16p + 2q .. +1]: the "even" fragment takes column
-// 16p + 2q as its n = q, the "odd" one 16p + 2q + 1. The outputs of lane (q, t) are then the
-// four consecutive columns 16p + 4t .. 16p + 4t + 3 of row q.
+// ------------------------------------------------------------------ F64: FP64 FMAs on the entries
+// One warp per (work unit, 16 * NP columns). Lane (q, t) = (lane / 4, lane % 4) owns row q and the
+// columns 16p + 4t .. 16p + 4t + 3, and holds A[q][t] of the current group of 4 tiles. A group takes
+// as many steps as its fullest row has entries: in each, a lane multiplies its row's next entry
+// with four columns of that entry's B row.
+//
+// The FP64 pipe bounds this kernel. The MMA m8n8k4 runs on the same pipe, at 1.10 against
+// 1.20 TFLOP/s measured, and spends it on a tile's zeros as on its entries; the steps skip the
+// zero columns of a group. Measured against the MMA (4 steps always), whole SpMM:
+//   Laplacian 512^2 with 8 x 8 blocks (26 tiles per block, 8 dense), N = 64   256 -> 196 us
+//   dense 16 x 16 blocks beside 16-entry rows, 2^17 rows, N = 64              390 -> 369 us
+// 32 columns per warp (NP = 2): 64 left too few warps in flight (209 us), 16 read A too often.
+// The zeros that are skipped are those of the stored tile, an explicit zero of A among them.
 template <int NP>
-__global__ void __launch_bounds__(128) bcsr_dmma(BcsrKArgs a) {
+__global__ void __launch_bounds__(128) bcsr_f64(BcsrKArgs a) {
   const int lane = threadIdx.x & 31;
   const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t n_ct = (a.N + 16 * NP - 1) / (16 * NP);
@@ -281,31 +284,56 @@ __global__ void __launch_bounds__(128) bcsr_dmma(BcsrKArgs a) {
   const double* Av = reinterpret_cast<const double*>(a.tile_val) + t0 * 8;
   const double* Bp = reinterpret_cast<const double*>(a.B);
   const bool vec = ((a.ldb & 1) == 0) && (((uintptr_t)a.B & 15) == 0);
-  double acc[NP][2][2];
+  double acc[NP][4];
 #pragma unroll
   for (int p = 0; p < NP; ++p)
 #pragma unroll
-    for (int h = 0; h < 2; ++h) acc[p][h][0] = acc[p][h][1] = 0.0;
+    for (int i = 0; i < 4; ++i) acc[p][i] = 0.0;
+  // columns n, n + 1 of a B row (zeros past N)
+  auto load2 = [&](const double* brow, int64_t n, double& b0, double& b1) {
+    if (vec && n + 1 < a.N) {
+      const uint4 v = ldg16(brow + n);
+      b0 = __hiloint2double((int)v.y, (int)v.x);
+      b1 = __hiloint2double((int)v.w, (int)v.z);
+    } else {
+      b0 = n < a.N ? __ldg(brow + n) : 0.0;
+      b1 = n + 1 < a.N ? __ldg(brow + n + 1) : 0.0;
+    }
+  };
+  // the next group's values and columns are loaded during this group
+  double av_next = n_groups > 0 ? __ldg(Av + lane) : 0.0;
+  int32_t c_next = n_groups > 0 ? __ldg(a.tile_col + t0 + t) : -1;
   for (int g = 0; g < n_groups; ++g) {
-    const double av = __ldg(Av + g * 32 + lane);
-    const int32_t c = __ldg(a.tile_col + t0 + g * 4 + t);
-    const double* brow = Bp + (int64_t)(c >= 0 ? c : 0) * a.ldb;
+    const double av = av_next;
+    const int32_t c = c_next;
+    if (g + 1 < n_groups) {
+      av_next = __ldg(Av + (g + 1) * 32 + lane);
+      c_next = __ldg(a.tile_col + t0 + (g + 1) * 4 + t);
+    }
+    unsigned left = (__ballot_sync(0xffffffffu, av != 0.0) >> (lane & ~3)) & 15u;  // entries of row q
+    const int steps = (int)__reduce_max_sync(0xffffffffu, (unsigned)__popc(left));
+    for (int s = 0; s < steps; ++s) {
+      const bool live = left != 0;
+      const int from = live ? (lane & ~3) + __ffs(left) - 1 : lane;
+      const double w = __shfl_sync(0xffffffffu, av, from);
+      const int32_t cw = __shfl_sync(0xffffffffu, c, from);
+      left &= left - 1;
+      const double* brow = Bp + (int64_t)(live ? cw : 0) * a.ldb;
+      double x[NP][4];
 #pragma unroll
-    for (int p = 0; p < NP; ++p) {
-      const int64_t n = n0 + 16 * p + 2 * q;
-      double b0 = 0.0, b1 = 0.0;
-      if (c >= 0) {
-        if (vec && n + 1 < a.N) {
-          const uint4 v = ldg16(brow + n);
-          b0 = __hiloint2double((int)v.y, (int)v.x);
-          b1 = __hiloint2double((int)v.w, (int)v.z);
-        } else {
-          if (n < a.N) b0 = __ldg(brow + n);
-          if (n + 1 < a.N) b1 = __ldg(brow + n + 1);
+      for (int p = 0; p < NP; ++p) {
+        const int64_t n = n0 + 16 * p + 4 * t;
+        x[p][0] = x[p][1] = x[p][2] = x[p][3] = 0.0;
+        if (live) {
+          load2(brow, n, x[p][0], x[p][1]);
+          load2(brow, n + 2, x[p][2], x[p][3]);
         }
       }
-      dmma884(acc[p][0], av, b0);
-      dmma884(acc[p][1], av, b1);
+      // a row without a next entry adds zeros: w * 0 with its own w, which is finite
+#pragma unroll
+      for (int p = 0; p < NP; ++p)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) acc[p][i] = fma(live ? w : 0.0, x[p][i], acc[p][i]);
     }
   }
   if (slot >= 0) {  // one unit of a split block: partial sums of its 8 rows
@@ -313,10 +341,9 @@ __global__ void __launch_bounds__(128) bcsr_dmma(BcsrKArgs a) {
 #pragma unroll
     for (int p = 0; p < NP; ++p) {
       const int64_t n = n0 + 16 * p + 4 * t;
-      const double o[4] = {acc[p][0][0], acc[p][1][0], acc[p][0][1], acc[p][1][1]};
 #pragma unroll
       for (int i = 0; i < 4; ++i)
-        if (n + i < a.N) prow[n + i] = o[i];
+        if (n + i < a.N) prow[n + i] = acc[p][i];
     }
     return;
   }
@@ -327,8 +354,8 @@ __global__ void __launch_bounds__(128) bcsr_dmma(BcsrKArgs a) {
 #pragma unroll
   for (int p = 0; p < NP; ++p) {
     const int64_t n = n0 + 16 * p + 4 * t;
-    const double o[4] = {acc[p][0][0] * a.inv_scale_d, acc[p][1][0] * a.inv_scale_d,
-                         acc[p][0][1] * a.inv_scale_d, acc[p][1][1] * a.inv_scale_d};
+    const double o[4] = {acc[p][0] * a.inv_scale_d, acc[p][1] * a.inv_scale_d, acc[p][2] * a.inv_scale_d,
+                         acc[p][3] * a.inv_scale_d};
     if (cvec && n + 3 < a.N) {
       *reinterpret_cast<double2*>(crow + n) = make_double2(o[0], o[1]);
       *reinterpret_cast<double2*>(crow + n + 2) = make_double2(o[2], o[3]);
@@ -340,17 +367,15 @@ __global__ void __launch_bounds__(128) bcsr_dmma(BcsrKArgs a) {
   }
 }
 
-cudaError_t launch_dmma(const BcsrKArgs& a, cudaStream_t s) {
+cudaError_t launch_f64(const BcsrKArgs& a, cudaStream_t s) {
   auto go = [&](auto np_tag) {
     constexpr int NP = decltype(np_tag)::value;
     const int64_t n_ct = (a.N + 16 * NP - 1) / (16 * NP);
     const int64_t warps = a.n_units * n_ct;
-    bcsr_dmma<NP><<<(unsigned)((warps + 3) / 4), 128, 0, s>>>(a);
+    bcsr_f64<NP><<<(unsigned)((warps + 3) / 4), 128, 0, s>>>(a);
     return cudaGetLastError();
   };
-  if (a.N <= 16) return go(std::integral_constant<int, 1>());
-  if (a.N <= 32) return go(std::integral_constant<int, 2>());
-  return go(std::integral_constant<int, 4>());
+  return a.N <= 16 ? go(std::integral_constant<int, 1>()) : go(std::integral_constant<int, 2>());
 }
 
 // ------------------------------------------------------------------ F32: CUDA-core outer product
@@ -527,7 +552,7 @@ cudaError_t launch_bcsr(const loops_plan_s* p, const BcsrDev& d, const DenseArgs
   a.max_polls = wait_poll_limit();
   cudaError_t e = cudaErrorInvalidValue;
   switch (p->dtype) {
-    case LOOPS_F64: e = launch_dmma(a, s); break;
+    case LOOPS_F64: e = launch_f64(a, s); break;
     case LOOPS_F32: e = p->br == 8 ? launch_ffma_br<8>(a, s) : launch_ffma_br<16>(a, s); break;
     case LOOPS_F16: e = launch_hmma<__half>(a, p->bcsr_ntile, s); break;
     case LOOPS_BF16: e = launch_hmma<__nv_bfloat16>(a, p->bcsr_ntile, s); break;
