@@ -8,6 +8,7 @@
 // shuffles; U B-row loads are kept in flight before their FMAs. Accumulation is in f64 for F64
 // and in f32 otherwise. Every output row has one writer; rows split in segments write partials
 // that a second kernel sums in segment order, so the result does not depend on scheduling.
+#include <cstring>
 #include <type_traits>
 
 #include "device_common.cuh"
@@ -49,6 +50,19 @@ __device__ __forceinline__ float out_scale<TrF16>(const CsrKArgs& a, int64_t n) 
 template <>
 __device__ __forceinline__ float out_scale<TrBF16>(const CsrKArgs& a, int64_t n) {
   return a.col_scale ? a.col_scale[n] * a.inv_scale_f : a.inv_scale_f;
+}
+
+// Accumulator value of an A value in its register form (Tr::TV).
+template <class Tr>
+__device__ __forceinline__ typename Tr::TAcc acc_value(typename Tr::TV v) {
+  if constexpr (sizeof(typename Tr::TB) == 2) {
+    const unsigned short u = (unsigned short)v;
+    typename Tr::TB x;
+    memcpy(&x, &u, 2);
+    return Tr::to_acc(x);
+  } else {
+    return v;
+  }
 }
 
 // A chunk of an item's entries, R per lane (entry r * G + sub): columns and values, zeros past the
@@ -223,76 +237,139 @@ __global__ void __launch_bounds__(kCsrThreads, (CsrShape<Tr, VPL>::kMinBlocks)) 
   store_item<Tr, G, VPL>(a, row, n0, ok, acc);
 }
 
-// Scalar path for any N and alignment: 32 lanes per item, one column per lane per pass.
-template <class Tr, int U>
-__global__ void __launch_bounds__(256) csr_spmm_scalar(CsrKArgs a) {
-  using TB = typename Tr::TB;
-  using TAcc = typename Tr::TAcc;
-  using TC = typename Tr::TC;
-  const int lane = threadIdx.x & 31;
-  const int64_t item = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32;
-  if (item >= a.n_items) return;
-  const int64_t beg = a.item_ptr[item];
-  const int64_t end = a.item_ptr[item + 1];
-  const int32_t row = a.item_row[item];
-  const int64_t n = (int64_t)blockIdx.y * 32 + lane;
-  const bool colok = n < a.N;
-  const TB* __restrict__ Bp = reinterpret_cast<const TB*>(a.B);
-  const TB* __restrict__ vals = reinterpret_cast<const TB*>(a.val);
-  TAcc acc = TAcc(0);
-  for (int64_t k0 = beg; k0 < end; k0 += 32) {
-    const int64_t k = k0 + lane;
-    int32_t c = 0;
-    TAcc v = TAcc(0);
-    if (k < end) {
-      c = __ldg(a.col + k);
-      v = Tr::to_acc(vals[k]);
-    }
-    const int cnt = (int)(end - k0 < 32 ? end - k0 : 32);
-    for (int j0 = 0; j0 < cnt; j0 += U) {
-      TAcc bv[U], av[U];
+// Path for any N and alignment: a group of G lanes per item, each lane with CP pieces of VW adjacent
+// columns (one load of VW elements where N and B's rows allow it), G pieces apart, so that a group
+// reads consecutive memory and a row of B in one pass. With loads of 2 to 8 bytes instructions
+// count first: few lanes with many pieces each (G = 8 up to 64 pieces per row) share an entry's
+// column, value and address over CP loads, waste few lanes on a ragged N, and let a warp take
+// several items. U entries with 8 to 24 elements in flight per lane, entries one chunk ahead.
+// 200,003-node graph, 4.1 M entries, N = 47, FP32: @ODD@, against 280 us with one column per lane
+// and the entries read per 32 columns, and 165 us with 32 lanes and two pieces.
+template <int CP, int VW>
+struct OddShape {
+  static constexpr int kInFlight = CP * VW <= 2 ? 8 : (CP * VW <= 6 ? 4 : 2);  // entries
+};
+
+// VW adjacent elements of a row of B, zeros when off
+template <class TB, int VW>
+__device__ __forceinline__ void load_piece(bool on, const TB* p, TB (&x)[VW]) {
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int j = j0 + u;
-        const int cj = __shfl_sync(0xffffffffu, c, j & 31);
-        av[u] = __shfl_sync(0xffffffffu, v, j & 31);
-        const bool ok = j < cnt && colok;
-        bv[u] = ok ? Tr::to_acc(Bp[(int64_t)cj * a.ldb + n]) : TAcc(0);
-        if (j >= cnt) av[u] = TAcc(0);
-      }
-#pragma unroll
-      for (int u = 0; u < U; ++u) acc = fma(av[u], bv[u], acc);
-    }
-  }
-  if (!colok) return;
-  if (row >= 0) {
-    TC* cp = reinterpret_cast<TC*>(a.C) + (int64_t)row * a.ldc + n;
-    const TC v = Tr::kScaled ? (TC)(acc * out_scale<Tr>(a, n)) : (TC)acc;
-    *cp = a.accumulate ? *cp + v : v;
+  for (int w = 0; w < VW; ++w) x[w] = TB(0);
+  if (!on) return;
+  if constexpr (VW == 1) {
+    x[0] = p[0];
+  } else if constexpr (VW * sizeof(TB) == 8) {
+    const uint2 v = __ldg(reinterpret_cast<const uint2*>(p));
+    memcpy(x, &v, 8);
   } else {
-    reinterpret_cast<TAcc*>(a.scratch)[(int64_t)(-1 - row) * a.N + n] = acc;
+    const unsigned v = __ldg(reinterpret_cast<const unsigned*>(p));
+    memcpy(x, &v, 4);
   }
 }
 
-// C[row, n] = scale_n * sum over the row's segments, in segment order.
-template <class Tr>
-__global__ void __launch_bounds__(256) split_reduce(const int32_t* __restrict__ split_row,
-                                                    const int32_t* __restrict__ slot_ptr,
-                                                    int64_t n_split, CsrKArgs a) {
+template <class Tr, int G, int CP, int VW>
+__global__ void __launch_bounds__(kCsrThreads) csr_spmm_odd(CsrKArgs a) {
+  using TB = typename Tr::TB;
   using TAcc = typename Tr::TAcc;
   using TC = typename Tr::TC;
-  const int64_t s = blockIdx.x;
-  if (s >= n_split) return;
+  using TV = typename Tr::TV;
+  constexpr int U = OddShape<CP, VW>::kInFlight;
+  static_assert(G % U == 0, "load batches tile the chunk of G entries");
+  const int lane = threadIdx.x & 31;
+  const int sub = lane & (G - 1);
+  const int64_t item = ((int64_t)blockIdx.x * kCsrThreads + threadIdx.x) / G;
+  if (item >= a.n_items) return;  // a group leaves as a whole
+  const unsigned gmask = (G == 32) ? 0xffffffffu : (((1u << G) - 1u) << (lane & ~(G - 1)));
+  const int64_t beg = a.item_ptr[item];
+  const int32_t len = (int32_t)(a.item_ptr[item + 1] - beg);
+  const int32_t row = a.item_row[item];
+  const int32_t n0 = (int32_t)blockIdx.y * (G * CP * VW) + sub * VW;  // piece i starts at column n0 + i * G * VW
+  bool ok[CP];
+#pragma unroll
+  for (int i = 0; i < CP; ++i) ok[i] = n0 + i * G * VW < (int32_t)a.N;
+  const TB* __restrict__ bl = reinterpret_cast<const TB*>(a.B) + n0;
+  TAcc acc[CP][VW];
+#pragma unroll
+  for (int i = 0; i < CP; ++i)
+#pragma unroll
+    for (int w = 0; w < VW; ++w) acc[i][w] = TAcc(0);
+  int32_t c[1], c_next[1];
+  TV v[1], v_next[1];
+  fetch_entries<Tr, G>(a, beg, len, 0, sub, c_next, v_next);
+  for (int32_t k0 = 0; k0 < len; k0 += G) {
+    c[0] = c_next[0];
+    v[0] = v_next[0];
+    fetch_entries<Tr, G>(a, beg, len, k0 + G, sub, c_next, v_next);
+    const int cnt = min(len - k0, G);  // uniform in the group
+    // entries past the chunk's end load nothing and carry zero values
+    auto batch = [&](int e0, auto tail_tag) {
+      constexpr bool TAIL = decltype(tail_tag)::value;
+      TB bv[U][CP][VW];
+      TAcc av[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int32_t cj = __shfl_sync(gmask, c[0], e0 + u, G);
+        av[u] = acc_value<Tr>(__shfl_sync(gmask, v[0], e0 + u, G));
+        const TB* brow = bl + (int64_t)cj * a.ldb;
+#pragma unroll
+        for (int i = 0; i < CP; ++i) load_piece<TB, VW>(ok[i] && (!TAIL || e0 + u < cnt), brow + i * G * VW, bv[u][i]);
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int i = 0; i < CP; ++i)
+#pragma unroll
+          for (int w = 0; w < VW; ++w) acc[i][w] = fma(av[u], Tr::to_acc(bv[u][i][w]), acc[i][w]);
+    };
+    int e0 = 0;
+    for (; e0 + U <= cnt; e0 += U) batch(e0, std::false_type());
+    if (e0 < cnt) batch(e0, std::true_type());
+  }
+#pragma unroll
+  for (int i = 0; i < CP; ++i) {
+    if (!ok[i]) continue;
+#pragma unroll
+    for (int w = 0; w < VW; ++w) {
+      const int32_t n = n0 + i * G * VW + w;
+      if (row >= 0) {
+        TC* cp = reinterpret_cast<TC*>(a.C) + (int64_t)row * a.ldc + n;
+        const TC o = Tr::kScaled ? (TC)(acc[i][w] * out_scale<Tr>(a, n)) : (TC)acc[i][w];
+        *cp = a.accumulate ? *cp + o : o;
+      } else {
+        reinterpret_cast<TAcc*>(a.scratch)[(int64_t)(-1 - row) * a.N + n] = acc[i][w];
+      }
+    }
+  }
+}
+
+// C[row, n] = scale_n * sum over the row's segments, in segment order, eight partials in flight.
+// Threads of a block cover columns x split rows, so that narrow rows fill the block.
+constexpr int kReduceThreads = 128;
+template <class Tr>
+__global__ void __launch_bounds__(kReduceThreads) split_reduce(const int32_t* __restrict__ split_row,
+                                                               const int32_t* __restrict__ slot_ptr,
+                                                               int64_t n_split, int log_tx, CsrKArgs a) {
+  using TAcc = typename Tr::TAcc;
+  using TC = typename Tr::TC;
+  const int64_t s = (int64_t)blockIdx.x * (kReduceThreads >> log_tx) + (threadIdx.x >> log_tx);
+  const int64_t n = ((int64_t)blockIdx.y << log_tx) + (threadIdx.x & ((1 << log_tx) - 1));
+  if (s >= n_split || n >= a.N) return;
   const int32_t row = split_row[s];
   const int32_t s0 = slot_ptr[s], s1 = slot_ptr[s + 1];
-  const TAcc* sc = reinterpret_cast<const TAcc*>(a.scratch);
-  for (int64_t n = (int64_t)blockIdx.y * blockDim.x + threadIdx.x; n < a.N; n += (int64_t)gridDim.y * blockDim.x) {
-    TAcc acc = TAcc(0);
-    for (int32_t q = s0; q < s1; ++q) acc += sc[(int64_t)q * a.N + n];
-    TC* cp = reinterpret_cast<TC*>(a.C) + (int64_t)row * a.ldc + n;
-    const TC v = Tr::kScaled ? (TC)(acc * out_scale<Tr>(a, n)) : (TC)acc;
-    *cp = a.accumulate ? *cp + v : v;
+  const TAcc* sc = reinterpret_cast<const TAcc*>(a.scratch) + n;
+  TAcc acc = TAcc(0);
+  int32_t q = s0;
+  for (; q + 8 <= s1; q += 8) {
+    TAcc x[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) x[i] = sc[(int64_t)(q + i) * a.N];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) acc += x[i];
   }
+  for (; q < s1; ++q) acc += sc[(int64_t)q * a.N];
+  TC* cp = reinterpret_cast<TC*>(a.C) + (int64_t)row * a.ldc + n;
+  const TC v = Tr::kScaled ? (TC)(acc * out_scale<Tr>(a, n)) : (TC)acc;
+  *cp = a.accumulate ? *cp + v : v;
 }
 
 // Backward of C = A . B in one pass over A^T: dB[j, :] = sum_i a_ij dC[i, :] and
@@ -492,6 +569,39 @@ cudaError_t launch_vec_g(const CsrKArgs& a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+template <class Tr, int VW>
+cudaError_t launch_odd_vw(const CsrKArgs& a, cudaStream_t s) {
+  const int64_t pieces = a.N / VW;
+  auto go = [&](auto g_tag, auto cp_tag) {
+    constexpr int G = decltype(g_tag)::value, CP = decltype(cp_tag)::value;
+    const dim3 grid((unsigned)((a.n_items * G + kCsrThreads - 1) / kCsrThreads),
+                    (unsigned)((pieces + G * CP - 1) / (G * CP)));
+    csr_spmm_odd<Tr, G, CP, VW><<<grid, kCsrThreads, 0, s>>>(a);
+    return cudaGetLastError();
+  };
+  using std::integral_constant;
+  using G8 = integral_constant<int, 8>;
+  if (pieces <= 8) return go(G8(), integral_constant<int, 1>());
+  if (pieces <= 16) return go(G8(), integral_constant<int, 2>());
+  if (pieces <= 24) return go(G8(), integral_constant<int, 3>());
+  if (pieces <= 32) return go(G8(), integral_constant<int, 4>());
+  if (pieces <= 48) return go(G8(), integral_constant<int, 6>());
+  if (pieces <= 64) return go(G8(), integral_constant<int, 8>());
+  if (pieces <= 96) return go(integral_constant<int, 16>(), integral_constant<int, 6>());
+  if (pieces <= 128) return go(integral_constant<int, 16>(), integral_constant<int, 8>());
+  return go(integral_constant<int, 32>(), integral_constant<int, 6>());
+}
+
+// Two columns per load where they divide N and every row of B keeps the load aligned.
+template <class Tr>
+cudaError_t launch_odd(const CsrKArgs& a, cudaStream_t s) {
+  constexpr int64_t eb = sizeof(typename Tr::TB);
+  if constexpr (eb <= 4) {
+    if (a.N % 2 == 0 && a.ldb % 2 == 0 && (uintptr_t)a.B % (2 * eb) == 0) return launch_odd_vw<Tr, 2>(a, s);
+  }
+  return launch_odd_vw<Tr, 1>(a, s);
+}
+
 CsrKArgs csr_args(const loops_plan_s* p, const CsrDev& d, const DenseArgs& da, bool accumulate) {
   CsrKArgs a;
   a.accumulate = accumulate ? 1 : 0;
@@ -516,8 +626,11 @@ CsrKArgs csr_args(const loops_plan_s* p, const CsrDev& d, const DenseArgs& da, b
 template <class Tr>
 cudaError_t launch_split_reduce(const CsrDev& d, const CsrKArgs& a, cudaStream_t s) {
   if (d.n_split == 0) return cudaSuccess;
-  dim3 grid((unsigned)d.n_split, (unsigned)std::min<int64_t>((a.N + 255) / 256, 64));
-  split_reduce<Tr><<<grid, 256, 0, s>>>(d.split_row, d.split_slot_ptr, d.n_split, a);
+  int log_tx = 0;  // threads along the columns: a power of two that covers them, up to the block
+  while ((1 << log_tx) < kReduceThreads && (1 << log_tx) < a.N) ++log_tx;
+  const int rows = kReduceThreads >> log_tx;
+  const dim3 grid((unsigned)((d.n_split + rows - 1) / rows), (unsigned)((a.N + (1 << log_tx) - 1) >> log_tx));
+  split_reduce<Tr><<<grid, kReduceThreads, 0, s>>>(d.split_row, d.split_slot_ptr, d.n_split, log_tx, a);
   return cudaGetLastError();
 }
 
@@ -550,9 +663,7 @@ cudaError_t launch_csr_t(const loops_plan_s* p, const CsrDev& d, const DenseArgs
         default: e = two ? launch_vec_g<Tr, 32, 2>(a, s) : launch_vec_g<Tr, 32, 1>(a, s); break;
       }
     } else {
-      dim3 grid((unsigned)((a.n_items * 32 + 255) / 256), (unsigned)((a.N + 31) / 32));
-      csr_spmm_scalar<Tr, 8><<<grid, 256, 0, s>>>(a);
-      e = cudaGetLastError();
+      e = launch_odd<Tr>(a, s);
     }
   }
   if (e == cudaSuccess) e = launch_split_reduce<Tr>(d, a, s);
