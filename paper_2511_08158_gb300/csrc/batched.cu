@@ -27,11 +27,12 @@
 #include "loops_internal.h"
 
 // Tuning knobs (compile time):
-// * resident blocks per SM the class kernels must allow (their register caps): CSR FP32, CSR
-//   16-bit, FFMA B_r 8, FFMA B_r 16 (its 64 accumulators per lane spill at 3 blocks);
-// * B-row loads in flight per lane in CSR items, FP32 and 16-bit (powers of two);
-// * tiles in flight in FFMA units, B_r 8 and B_r 16;
+// * resident blocks per SM the CSR class kernels must allow (their register caps), FP32 and
+//   16-bit, and their B-row loads in flight per lane (powers of two);
 // * cp.async stages of the HMMA units.
+// Measured on a batch of 128 matrices in FP32 (723 us) and 96 in BF16 (355 us): FP32 CSR with four
+// loads at 4 or 5 blocks 3 and 7 % slower; 16-bit CSR at 3 or 5 blocks, or with 2 or 8 loads, 6 to
+// 17 %; HMMA with 2 or 4 stages within 2 %.
 #ifndef LOOPS_BATCHED_CSR_MIN_BLOCKS
 #define LOOPS_BATCHED_CSR_MIN_BLOCKS 3
 #endif
@@ -48,20 +49,8 @@ static_assert(LOOPS_BATCHED_CSR16_LOADS >= 1 && (LOOPS_BATCHED_CSR16_LOADS & (LO
               "16-bit CSR loads in flight must be a power of two");
 static_assert(LOOPS_BATCHED_CSR_LOADS >= 2 && (LOOPS_BATCHED_CSR_LOADS & (LOOPS_BATCHED_CSR_LOADS - 1)) == 0,
               "CSR loads in flight must be a power of two: the load batches tile a chunk exactly");
-#ifndef LOOPS_BATCHED_FFMA_TILES
-#define LOOPS_BATCHED_FFMA_TILES 4
-#endif
 #ifndef LOOPS_BATCHED_HMMA_STAGES
 #define LOOPS_BATCHED_HMMA_STAGES 3
-#endif
-#ifndef LOOPS_BATCHED_FFMA_MIN_BLOCKS
-#define LOOPS_BATCHED_FFMA_MIN_BLOCKS 3
-#endif
-#ifndef LOOPS_BATCHED_FFMA16_MIN_BLOCKS
-#define LOOPS_BATCHED_FFMA16_MIN_BLOCKS 2
-#endif
-#ifndef LOOPS_BATCHED_FFMA16_TILES
-#define LOOPS_BATCHED_FFMA16_TILES 2
 #endif
 
 namespace loops {
@@ -111,7 +100,7 @@ __device__ __forceinline__ int64_t claim(unsigned long long* counter, int lane) 
 // the 16-byte column vectors p * G + sub (p < VPL). Entries are read R per lane at a time
 // (chunks of G * R entries, broadcast by shuffles), and the next chunk's entries are loaded
 // while the current chunk's B rows are in flight.
-template <class Tr, int G, int VPL>
+template <class Tr, int G, int VPL, bool FULL>
 __device__ __forceinline__ void csr_item(const BatchDesc& d, int64_t item, int sub, unsigned gmask) {
   using TB = typename Tr::TB;
   using TAcc = typename Tr::TAcc;
@@ -139,7 +128,7 @@ __device__ __forceinline__ void csr_item(const BatchDesc& d, int64_t item, int s
 #pragma unroll
   for (int p = 0; p < VPL; ++p) {
     const int32_t off = (p * G + sub) * VE;
-    colok[p] = off < N;
+    colok[p] = FULL || off < N;
     bl[p] = reinterpret_cast<const TB*>(d.B) + off;
   }
   TAcc acc[VPL][VE];
@@ -178,7 +167,10 @@ __device__ __forceinline__ void csr_item(const BatchDesc& d, int64_t item, int s
           const uint32_t cj = (uint32_t)__shfl_sync(gmask, c[e / G], e % G, G);
           av[u] = __shfl_sync(gmask, v[e / G], e % G, G);
 #pragma unroll
-          for (int p = 0; p < VPL; ++p) bv[u][p] = colok[p] ? ldg16(bl[p] + cj * ldb) : make_uint4(0, 0, 0, 0);
+          for (int p = 0; p < VPL; ++p) {
+            if constexpr (FULL) bv[u][p] = ldg16(bl[p] + cj * ldb);
+            else bv[u][p] = ldg16_if(colok[p], bl[p] + cj * ldb);
+          }
         }
 #pragma unroll
         for (int u = 0; u < U; ++u)
@@ -247,7 +239,7 @@ constexpr int csr_min_blocks() {
   return Tr::kVE == 8 ? LOOPS_BATCHED_CSR16_MIN_BLOCKS : LOOPS_BATCHED_CSR_MIN_BLOCKS;
 }
 
-template <class Tr, int G, int VPL>
+template <class Tr, int G, int VPL, bool FULL>
 __global__ void __launch_bounds__(256, csr_min_blocks<Tr>()) batched_csr(const BatchDesc* __restrict__ descs,
                                                       const BatchTask* __restrict__ tasks, int64_t n_tasks,
                                                       unsigned long long* counter) {
@@ -257,24 +249,36 @@ __global__ void __launch_bounds__(256, csr_min_blocks<Tr>()) batched_csr(const B
   for (int64_t t = claim(counter, lane); t < n_tasks; t = claim(counter, lane)) {
     const BatchTask task = tasks[t];
     const BatchDesc& d = descs[task.m];
-    for (int32_t i = grp; i < task.count; i += 32 / G) csr_item<Tr, G, VPL>(d, task.first + i, sub, gmask);
+    for (int32_t i = grp; i < task.count; i += 32 / G) csr_item<Tr, G, VPL, FULL>(d, task.first + i, sub, gmask);
   }
 }
 
 // ------------------------------------------------------------------ F32 BCSR units
+// Tiles in flight and resident blocks per SM (register caps). The units wait on their loads: with
+// B_r 8 two tiles at 4 blocks beat four at 3 (batch of 128 matrices 755 -> 724 us, with the
+// unpredicated loads; N = 16, 32, 64 of the 512-matrix batch 119, 234, 352 -> 112, 222, 323 us) and
+// three at either; one tile, or two at 5 blocks, spill (1.4x the call). B_r 16 holds 64
+// accumulators per lane: two tiles at 2 blocks.
+constexpr int kFfmaTiles = 2;
+template <int BR>
+struct FfmaShape {
+  static constexpr int kMinBlocks = BR == 16 ? 2 : 4;
+};
+
 // One F32 BCSR unit (B_r rows, tile-major values) for a group of G lanes, 4 columns per lane;
 // T tiles' B vectors and A values are loaded before their FMAs.
-template <int BR, int G>
+template <int BR, int G, bool FULL>
 __device__ __forceinline__ void ffma_unit(const BatchDesc& d, int64_t u, int sub) {
-  constexpr int T = BR == 8 ? LOOPS_BATCHED_FFMA_TILES : LOOPS_BATCHED_FFMA16_TILES;
+  constexpr int T = kFfmaTiles;
   const int32_t b = d.unit_block[u];
   const int64_t rb = d.rb_id[b];
   const int64_t t0 = d.unit_t0[u], t1 = d.unit_t1[u];
   const int32_t slot = d.unit_slot[u];
   const float* __restrict__ Av = reinterpret_cast<const float*>(d.tile_val);
-  const float* __restrict__ Bp = reinterpret_cast<const float*>(d.B);
   const int64_t n = (int64_t)sub * 4;
-  const bool colok = n < d.N;
+  const bool colok = FULL || n < d.N;
+  const float* __restrict__ bl = reinterpret_cast<const float*>(d.B) + n;
+  const uint32_t ldb = (uint32_t)d.ldb;  // the batched call keeps every B below 2^31 elements
   float acc[BR][4];
 #pragma unroll
   for (int r = 0; r < BR; ++r)
@@ -298,8 +302,15 @@ __device__ __forceinline__ void ffma_unit(const BatchDesc& d, int64_t u, int sub
 #pragma unroll
     for (int q = 0; q < T; ++q) cc[q] = base + q < t1 ? __ldg(d.tile_col + base + q) : -1;
   };
-  auto load_tile = [&](bool live, int64_t tt, int32_t c, uint4& v, uint4 (&w)[BR / 4]) {
-    v = ldg16_if(live && c >= 0 && colok, Bp + (int64_t)c * d.ldb + n);
+  // F32 blocks have no padding tiles, so every tile of a full batch has a column
+  auto load_tile = [&](int64_t tt, int32_t c, uint4& v, uint4 (&w)[BR / 4]) {
+    if constexpr (FULL) v = ldg16(bl + (uint32_t)c * ldb);
+    else v = ldg16_if(colok, bl + (uint32_t)c * ldb);
+#pragma unroll
+    for (int r4 = 0; r4 < BR / 4; ++r4) w[r4] = ldg16(Av + tt * BR + r4 * 4);
+  };
+  auto load_tile_if = [&](bool live, int64_t tt, int32_t c, uint4& v, uint4 (&w)[BR / 4]) {
+    v = ldg16_if(live && colok, bl + (uint32_t)c * ldb);
 #pragma unroll
     for (int r4 = 0; r4 < BR / 4; ++r4) w[r4] = ldg16_if(live, Av + tt * BR + r4 * 4);
   };
@@ -312,7 +323,7 @@ __device__ __forceinline__ void ffma_unit(const BatchDesc& d, int64_t u, int sub
     uint4 v[T];
     uint4 w[T][BR / 4];
 #pragma unroll
-    for (int q = 0; q < T; ++q) load_tile(true, tt + q, c[q], v[q], w[q]);
+    for (int q = 0; q < T; ++q) load_tile(tt + q, c[q], v[q], w[q]);
 #pragma unroll
     for (int q = 0; q < T; ++q) tile_fma(v[q], w[q]);
 #pragma unroll
@@ -322,7 +333,7 @@ __device__ __forceinline__ void ffma_unit(const BatchDesc& d, int64_t u, int sub
     uint4 v[T];
     uint4 w[T][BR / 4];
 #pragma unroll
-    for (int q = 0; q < T; ++q) load_tile(tt + q < t1, tt + q, c[q], v[q], w[q]);
+    for (int q = 0; q < T; ++q) load_tile_if(tt + q < t1, tt + q, c[q], v[q], w[q]);
 #pragma unroll
     for (int q = 0; q < T; ++q) tile_fma(v[q], w[q]);
   }
@@ -343,8 +354,8 @@ __device__ __forceinline__ void ffma_unit(const BatchDesc& d, int64_t u, int sub
   }
 }
 
-template <int BR, int G>
-__global__ void __launch_bounds__(256, BR == 8 ? LOOPS_BATCHED_FFMA_MIN_BLOCKS : LOOPS_BATCHED_FFMA16_MIN_BLOCKS)
+template <int BR, int G, bool FULL>
+__global__ void __launch_bounds__(256, FfmaShape<BR>::kMinBlocks)
     batched_ffma(const BatchDesc* __restrict__ descs,
                                                        const BatchTask* __restrict__ tasks, int64_t n_tasks,
                                                        unsigned long long* counter) {
@@ -353,7 +364,7 @@ __global__ void __launch_bounds__(256, BR == 8 ? LOOPS_BATCHED_FFMA_MIN_BLOCKS :
   for (int64_t t = claim(counter, lane); t < n_tasks; t = claim(counter, lane)) {
     const BatchTask task = tasks[t];
     const BatchDesc& d = descs[task.m];
-    for (int32_t i = grp; i < task.count; i += 32 / G) ffma_unit<BR, G>(d, task.first + i, sub);
+    for (int32_t i = grp; i < task.count; i += 32 / G) ffma_unit<BR, G, FULL>(d, task.first + i, sub);
   }
 }
 
@@ -379,19 +390,30 @@ __device__ __forceinline__ void hmma_unit(const BatchDesc& d, int64_t u, T* sB, 
   const int32_t slot = d.unit_slot[u];
   const int N = (int)d.N;
   const T* Bp = reinterpret_cast<const T*>(d.B);
+  const uint32_t ldb = (uint32_t)d.ldb;  // the batched call keeps every B below 2^31 elements
   const uint4* Af = reinterpret_cast<const uint4*>(d.tile_val) + (t0 / 16) * 32;
   const int q = lane >> 2, t = lane & 3;
   for (int c0 = 0; c0 < N; c0 += kHChunk) {
     const int NC = min(kHChunk, N - c0);   // columns of this chunk (a multiple of 8)
     const int NF = NC / 8;
     // stage of group g: this lane copies the vectors i = lane, lane + 32, ... of its 16 x NF
-    // piece (column -1: zero-filled, nothing read)
+    // piece (column -1: zero-filled, nothing read). Groups are issued in order, and lane k % 16
+    // holds the column of tile k of the next one, loaded when the one before it was issued, so
+    // that no copy waits on its column.
+    const int sh = 31 - __clz(NF);
+    const bool pow2 = (NF & (NF - 1)) == 0;
+    const int32_t* cols = d.tile_col + t0 + (lane & 15);
+    int32_t c_next = n_groups > 0 ? __ldg(cols) : -1;
     auto issue = [&](int g) {
       T* st = sB + (g % kHStages) * kHStageElems;
-      for (int i = lane; i < 16 * NF; i += 32) {
-        const int k = i / NF, qv = i - k * NF;
-        const int32_t c = __ldg(d.tile_col + t0 + g * 16 + k);
-        const T* src = c >= 0 ? Bp + (int64_t)c * d.ldb + c0 + qv * 8 : Bp;
+      const int32_t c_mine = c_next;
+      if (g + 1 < n_groups) c_next = __ldg(cols + (g + 1) * 16);
+      for (int i0 = 0; i0 < 16 * NF; i0 += 32) {
+        const int i = i0 + lane;
+        const int k = pow2 ? i >> sh : i / NF, qv = i - k * NF;
+        const int32_t c = __shfl_sync(0xffffffffu, c_mine, k & 15);
+        if (i >= 16 * NF) continue;
+        const T* src = c >= 0 ? Bp + (uint32_t)c * ldb + c0 + qv * 8 : Bp;
         cp_async16(st + k * kHStride + qv * 8, src, c >= 0 ? 16 : 0);
       }
     };
@@ -523,52 +545,47 @@ __global__ void __launch_bounds__(256) batched_bsplit_reduce(const BatchDesc* __
 // ------------------------------------------------------------------ class dispatch
 using ClassKernel = void (*)(const BatchDesc*, const BatchTask*, int64_t, unsigned long long*);
 
-template <class Tr>
+template <class Tr, bool FULL>
 ClassKernel csr_kernel(int G, int VPL) {
   // 16-bit rows (N <= 128) take one vector per lane: at most 16 lanes, never two vectors
   if constexpr (Tr::kVE == 8) {
     switch (VPL == 1 ? G : 0) {
-      case 1: return batched_csr<Tr, 1, 1>;
-      case 2: return batched_csr<Tr, 2, 1>;
-      case 4: return batched_csr<Tr, 4, 1>;
-      case 8: return batched_csr<Tr, 8, 1>;
-      case 16: return batched_csr<Tr, 16, 1>;
+      case 1: return batched_csr<Tr, 1, 1, FULL>;
+      case 2: return batched_csr<Tr, 2, 1, FULL>;
+      case 4: return batched_csr<Tr, 4, 1, FULL>;
+      case 8: return batched_csr<Tr, 8, 1, FULL>;
+      case 16: return batched_csr<Tr, 16, 1, FULL>;
       default: return nullptr;
     }
   } else {
     if (VPL == 2) {
       switch (G) {
-        case 8: return batched_csr<Tr, 8, 2>;
-        case 16: return batched_csr<Tr, 16, 2>;
+        case 8: return batched_csr<Tr, 8, 2, FULL>;
+        case 16: return batched_csr<Tr, 16, 2, FULL>;
         default: return nullptr;
       }
     }
     switch (G) {
-      case 1: return batched_csr<Tr, 1, 1>;
-      case 2: return batched_csr<Tr, 2, 1>;
-      case 4: return batched_csr<Tr, 4, 1>;
-      case 8: return batched_csr<Tr, 8, 1>;
-      case 16: return batched_csr<Tr, 16, 1>;
-      case 32: return batched_csr<Tr, 32, 1>;
+      case 1: return batched_csr<Tr, 1, 1, FULL>;
+      case 2: return batched_csr<Tr, 2, 1, FULL>;
+      case 4: return batched_csr<Tr, 4, 1, FULL>;
+      case 8: return batched_csr<Tr, 8, 1, FULL>;
+      case 16: return batched_csr<Tr, 16, 1, FULL>;
+      case 32: return batched_csr<Tr, 32, 1, FULL>;
       default: return nullptr;
     }
   }
 }
 
-template <int BR, int G>
-ClassKernel ffma_g(int*, int*) {
-  return batched_ffma<BR, G>;
-}
-
-template <int BR>
-ClassKernel ffma_kernel(int G, int* smem, int* threads) {
+template <int BR, bool FULL>
+ClassKernel ffma_kernel(int G) {
   switch (G) {
-    case 1: return ffma_g<BR, 1>(smem, threads);
-    case 2: return ffma_g<BR, 2>(smem, threads);
-    case 4: return ffma_g<BR, 4>(smem, threads);
-    case 8: return ffma_g<BR, 8>(smem, threads);
-    case 16: return ffma_g<BR, 16>(smem, threads);
-    case 32: return ffma_g<BR, 32>(smem, threads);
+    case 1: return batched_ffma<BR, 1, FULL>;
+    case 2: return batched_ffma<BR, 2, FULL>;
+    case 4: return batched_ffma<BR, 4, FULL>;
+    case 8: return batched_ffma<BR, 8, FULL>;
+    case 16: return batched_ffma<BR, 16, FULL>;
+    case 32: return batched_ffma<BR, 32, FULL>;
     default: return nullptr;
   }
 }
@@ -579,15 +596,16 @@ ClassKernel class_kernel(loops_dtype dtype, const BatchClass& c, int* smem, int*
   *threads = 256;
   if (c.kind == 0) {
     switch (dtype) {
-      case LOOPS_F32: return csr_kernel<TrF32>(c.G, c.vpl);
-      case LOOPS_F16: return csr_kernel<TrF16>(c.G, c.vpl);
-      case LOOPS_BF16: return csr_kernel<TrBF16>(c.G, c.vpl);
+      case LOOPS_F32: return c.full ? csr_kernel<TrF32, true>(c.G, c.vpl) : csr_kernel<TrF32, false>(c.G, c.vpl);
+      case LOOPS_F16: return c.full ? csr_kernel<TrF16, true>(c.G, c.vpl) : csr_kernel<TrF16, false>(c.G, c.vpl);
+      case LOOPS_BF16: return c.full ? csr_kernel<TrBF16, true>(c.G, c.vpl) : csr_kernel<TrBF16, false>(c.G, c.vpl);
       default: return nullptr;
     }
   }
   if (c.kind == 1) {
     if (dtype != LOOPS_F32) return nullptr;
-    return c.br == 8 ? ffma_kernel<8>(c.G, smem, threads) : ffma_kernel<16>(c.G, smem, threads);
+    if (c.full) return c.br == 8 ? ffma_kernel<8, true>(c.G) : ffma_kernel<16, true>(c.G);
+    return c.br == 8 ? ffma_kernel<8, false>(c.G) : ffma_kernel<16, false>(c.G);
   }
   *smem = kHmmaSmemPerWarp * 8;
   if (dtype == LOOPS_F16) return batched_hmma<__half>;

@@ -174,9 +174,11 @@ void csr_shape(loops_dtype dtype, int64_t N, int32_t* G, int32_t* vpl) {
   *G = next_pow2(*vpl == 2 ? (nvec + 1) / 2 : nvec);
 }
 
-// Class key: kind, then group width, then vectors per lane (CSR) or tile height (F32 BCSR,
-// 8 or 16, stored as 8 -> 8, 16 -> 0 in the low four bits).
-int64_t class_key(int32_t kind, int32_t G, int32_t low) { return ((int64_t)kind << 16) | (G << 4) | (low & 0xf); }
+// Class key: kind, then group width, then whether the group's vectors cover N exactly, then vectors
+// per lane (CSR) or tile height (F32 BCSR, 8 or 16, stored as 8 -> 8, 16 -> 0 in the low four bits).
+int64_t class_key(int32_t kind, int32_t G, bool full, int32_t low) {
+  return ((int64_t)kind << 16) | (G << 5) | ((full ? 1 : 0) << 4) | (low & 0xf);
+}
 
 // Builds the sub-plan of matrix m for the given options, tile height and threshold.
 using SubBuilder = std::function<loops_status(int32_t m, const loops_plan_opts& o, int32_t br, double tau,
@@ -239,7 +241,7 @@ loops_status build_batch(const loops_csr* As, const int64_t* Ns, int32_t count, 
       }
       tasks.push_back({m, 0, i, (int32_t)(j - i), 0});
       cost.push_back((double)(nnz + (j - i)) * (double)N);
-      cls.push_back(class_key(0, G, vpl));
+      cls.push_back(class_key(0, G, N == (int64_t)G * vpl * VE, vpl));
       i = j;
     }
     // BCSR units (most tiles first): F32 in groups of G lanes (4 columns each), 16-bit one per warp
@@ -251,13 +253,13 @@ loops_status build_batch(const loops_csr* As, const int64_t* Ns, int32_t count, 
         const int32_t cnt = (int32_t)std::min<int64_t>(rf, bd.n_units - q);
         tasks.push_back({m, 1, q, cnt, 0});
         cost.push_back((double)bd.h_unit_tiles[(size_t)q] * br * (double)N);
-        cls.push_back(class_key(1, Gf, br));
+        cls.push_back(class_key(1, Gf, N == (int64_t)Gf * VE, br));
       }
     } else {
       for (int64_t q = 0; q < bd.n_units; ++q) {
         tasks.push_back({m, 2, q, 1, 0});
         cost.push_back((double)bd.h_unit_tiles[(size_t)q] * br * (double)N);
-        cls.push_back(class_key(2, 0, 0));
+        cls.push_back(class_key(2, 0, false, 0));
       }
     }
     for (int64_t sidx = 0; sidx < bd.n_split; ++sidx) bsplits.push_back(make_int2(m, (int)sidx));
@@ -283,7 +285,8 @@ loops_status build_batch(const loops_csr* As, const int64_t* Ns, int32_t count, 
     while (j < idx.size() && cls[(size_t)idx[j]] == key) ++j;
     BatchClass bc;
     bc.kind = (int32_t)(key >> 16);
-    bc.G = (int32_t)((key >> 4) & 0xfff);
+    bc.G = (int32_t)((key >> 5) & 0x7ff);
+    bc.full = (int32_t)((key >> 4) & 1);
     bc.vpl = bc.kind == 0 ? (int32_t)(key & 0xf) : 1;
     bc.br = (bc.kind == 1 && (key & 0xf) == 8) ? 8 : 16;
     bc.first = (int64_t)i;

@@ -262,6 +262,7 @@ struct BatchClass {
   int32_t G;
   int32_t vpl;
   int32_t br;                          // tile height of an F32 BCSR class (8 or 16)
+  int32_t full;                        // the lanes' vectors cover N exactly (unpredicated loads)
   int32_t grid;
   int64_t first;
   int64_t n_tasks;
