@@ -271,16 +271,19 @@ static loops_plan_s* new_plan(int64_t n_rows, int64_t n_cols, int64_t nnz, int64
   return p;
 }
 
-// Error word, side stream and fork/join events of a plan that runs SpMM calls.
+// What the SpMM calls of a plan need besides its arrays: the error word of the BCSR kernels, and a
+// side stream with fork/join events where both parts run. An all-CSR plan needs none of them.
 static loops_status plan_runtime(loops_plan_s* p) {
+  if (p->dev.bcsr.n_rb == 0) return LOOPS_OK;
   cudaError_t e = dev_malloc((void**)&p->d_error, sizeof(int32_t));
   if (e == cudaSuccess) e = cudaMemset(p->d_error, 0, sizeof(int32_t));
-  if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&p->side, cudaStreamNonBlocking);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->ev_fork, cudaEventDisableTiming);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->ev_join, cudaEventDisableTiming);
-  if (e != cudaSuccess) return cuda_status(e, "plan setup");
-  p->other_bytes += sizeof(int32_t);
-  return LOOPS_OK;
+  if (e == cudaSuccess) p->other_bytes += sizeof(int32_t);
+  if (e == cudaSuccess && p->dev.csr.n_items > 0) {
+    e = cudaStreamCreateWithFlags(&p->side, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->ev_fork, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->ev_join, cudaEventDisableTiming);
+  }
+  return e == cudaSuccess ? LOOPS_OK : cuda_status(e, "plan setup");
 }
 
 loops_status make_plan(const loops_csr* A, const double* vals, int64_t N, loops_dtype dtype,
@@ -1319,17 +1322,17 @@ loops_status loops_plan_check(loops_plan_t p, loops_stream_t stream) {
   if (st) return st;
   int32_t h = 0;
   cudaStream_t s = (cudaStream_t)stream;
-  cudaError_t e = cudaMemcpyAsync(&h, p->d_error, sizeof(int32_t), cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(p->d_error, 0, sizeof(int32_t), s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  if (e != cudaSuccess) return cuda_status(e, "read error word");
-  if (p->transposed) {
-    int32_t ht = 0;
-    e = cudaMemcpyAsync(&ht, p->transposed->d_error, sizeof(int32_t), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(p->transposed->d_error, 0, sizeof(int32_t), s);
+  for (const loops_plan_s* q : {(const loops_plan_s*)p, (const loops_plan_s*)p->transposed}) {
+    if (!q) continue;
+    int32_t hq = 0;
+    cudaError_t e = cudaSuccess;
+    if (q->d_error) {  // none without a BCSR part: no kernel of the plan waits
+      e = cudaMemcpyAsync(&hq, q->d_error, sizeof(int32_t), cudaMemcpyDeviceToHost, s);
+      if (e == cudaSuccess) e = cudaMemsetAsync(q->d_error, 0, sizeof(int32_t), s);
+    }
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return cuda_status(e, "read error word");
-    h |= ht;
+    h |= hq;
   }
   if (h & kErrWaitTimeout) {
     set_error("a device-side wait exceeded its bound");

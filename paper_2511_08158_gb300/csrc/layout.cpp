@@ -226,13 +226,17 @@ loops_status upload_part(loops_plan_s* p, int64_t N) {
 }
 
 void free_part(PartDev& d) {
-  void* ptrs[] = {d.csr.item_row, d.csr.item_ptr, d.csr.col, d.csr.val, d.csr.split_row,
-                  d.csr.split_slot_ptr, d.csr.scratch, d.csr_acc.item_row, d.csr_acc.item_ptr,
-                  d.csr_acc.col, d.csr_acc.val, d.csr_acc.split_row, d.csr_acc.split_slot_ptr,
-                  d.csr_acc.scratch, d.bcsr.rb_id, d.bcsr.rb_ptr,
-                  d.bcsr.tile_col, d.bcsr.tile_val, d.bcsr.unit_block, d.bcsr.unit_t0,
-                  d.bcsr.unit_t1, d.bcsr.unit_slot, d.bcsr.split_block, d.bcsr.split_slot_ptr,
-                  d.bcsr.scratch};
+  for (CsrDev* c : {&d.csr, &d.csr_acc}) {
+    if (c->slab) {
+      cudaFree(c->slab);
+      continue;
+    }
+    void* ptrs[] = {c->item_row, c->item_ptr, c->col, c->val, c->split_row, c->split_slot_ptr, c->scratch};
+    for (void* q : ptrs)
+      if (q) cudaFree(q);
+  }
+  void* ptrs[] = {d.bcsr.rb_id, d.bcsr.rb_ptr, d.bcsr.tile_col, d.bcsr.tile_val, d.bcsr.unit_block, d.bcsr.unit_t0,
+                  d.bcsr.unit_t1, d.bcsr.unit_slot, d.bcsr.split_block, d.bcsr.split_slot_ptr, d.bcsr.scratch};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   d = PartDev();
@@ -312,7 +316,7 @@ loops_status upload_value_maps(loops_plan_s* p, const std::vector<int64_t>* rema
 }
 
 void free_value_maps(ValueMapDev& m) {
-  void* ptrs[] = {m.csr_src, m.bcsr_ptr, m.bcsr_src};
+  void* ptrs[] = {m.csr_src_in_slab ? nullptr : m.csr_src, m.bcsr_ptr, m.bcsr_src};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   m = ValueMapDev();

@@ -145,6 +145,7 @@ struct CsrDev {
   int32_t* split_row = nullptr;        // global C row of each split row
   int32_t* split_slot_ptr = nullptr;   // size n_split + 1
   void* scratch = nullptr;             // n_slots x N partial sums (accumulator type)
+  void* slab = nullptr;                // when set, the one allocation that holds the arrays above
   // host mirrors used for export
   std::vector<int32_t> h_item_row;
   std::vector<int64_t> h_item_ptr;
@@ -208,6 +209,7 @@ struct SddmmDev {
 struct ValueMapDev {
   int64_t n_csr = 0, n_slots = 0;
   bool wide = false;
+  bool csr_src_in_slab = false;        // csr_src lies in the CSR part's slab
   void* csr_src = nullptr;
   void* bcsr_ptr = nullptr;
   void* bcsr_src = nullptr;
@@ -321,8 +323,8 @@ struct loops_plan_s {
   loops::SddmmDev sddmm;
   loops::ValueMapDev vmap;
   std::vector<int64_t> t_perm;         // A^T entry e comes from input entry t_perm[e]
-  int32_t* d_error;                    // device error word
-  cudaStream_t side;                   // second stream for the BCSR part
+  int32_t* d_error;                    // device error word (plans with a BCSR part)
+  cudaStream_t side;                   // second stream for the BCSR part, beside a CSR part
   cudaEvent_t ev_fork, ev_join;
   void* stage_B;                       // loops_spmm_host staging buffers
   void* stage_C;

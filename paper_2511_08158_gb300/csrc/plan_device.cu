@@ -52,22 +52,66 @@ __device__ int g_build_err;
 // ------------------------------------------------------------------ temporaries
 // Device allocations that live for one build: stream-ordered (the device's memory pool, no
 // device-wide synchronisation per allocation), released on the build's stream when the arena
-// goes out of scope.
+// goes out of scope. Small arrays share chunks: the pool maps and unmaps memory per allocation
+// (about 15 us each at the synchronisation that follows their release).
 struct Arena {
+  static constexpr size_t kChunkBytes = (size_t)4 << 20, kAlign = 256;
   std::vector<void*> ptrs;
+  char* chunk = nullptr;
+  size_t chunk_left = 0;
   cudaStream_t s = nullptr;
   cudaError_t err = cudaSuccess;
   template <class T>
   T* get(int64_t n) {
     if (err != cudaSuccess) return nullptr;
+    const size_t bytes = ((size_t)std::max<int64_t>(n, 1) * sizeof(T) + kAlign - 1) / kAlign * kAlign;
+    if (bytes <= chunk_left) {
+      T* q = (T*)chunk;
+      chunk += bytes;
+      chunk_left -= bytes;
+      return q;
+    }
     void* q = nullptr;
-    err = dev_malloc_async(&q, (size_t)std::max<int64_t>(n, 1) * sizeof(T), s);
+    const size_t take = std::max(bytes, kChunkBytes);
+    err = dev_malloc_async(&q, take, s);
     if (err != cudaSuccess) { cudaGetLastError(); return nullptr; }
     ptrs.push_back(q);
+    if (take - bytes > chunk_left) {  // keep filling the emptier chunk
+      chunk = (char*)q + bytes;
+      chunk_left = take - bytes;
+    }
     return (T*)q;
   }
   ~Arena() {
     for (void* q : ptrs) cudaFreeAsync(q, s);
+  }
+};
+
+// Several plan-owned arrays in one device allocation (cudaMalloc and cudaFree cost 20 to 60 us each):
+// add() them, then alloc().
+struct Slab {
+  struct Part {
+    void** dst;
+    size_t bytes;
+  };
+  std::vector<Part> parts;
+  template <class T>
+  void add(T** dst, int64_t n) {
+    if (n > 0) parts.push_back({(void**)dst, ((size_t)n * sizeof(T) + 255) / 256 * 256});
+  }
+  cudaError_t alloc(void** base, int64_t& bytes) {
+    size_t total = 0;
+    for (const Part& p : parts) total += p.bytes;
+    if (total == 0) return cudaSuccess;
+    cudaError_t e = dev_malloc(base, total);
+    if (e != cudaSuccess) { cudaGetLastError(); *base = nullptr; return e; }
+    bytes += (int64_t)total;
+    char* at = (char*)*base;
+    for (const Part& p : parts) {
+      *p.dst = at;
+      at += p.bytes;
+    }
+    return cudaSuccess;
   }
 };
 
@@ -983,34 +1027,31 @@ loops_status build_csr_set(loops_plan_s* p, const DevCsrIn& A, const int64_t* re
   int64_t* pre_len = ar.get<int64_t>(n_it);
   int64_t* dlen = ar.get<int64_t>(n_it + 1);
   NEED(dlen);
-  if (total.splits) {
-    TRY(own(&cd.split_row, total.splits, bytes));
-    TRY(own(&cd.split_slot_ptr, total.splits + 1, bytes));
-  }
+  const int64_t es = dense_elem_bytes(p->dtype), acc_bytes = p->dtype == LOOPS_F64 ? 8 : 4;
+  Slab slab;
+  slab.add(&cd.item_row, n_it);
+  slab.add(&cd.item_ptr, n_it + 1);
+  slab.add(&cd.col, n_canon);
+  slab.add((uint8_t**)&cd.val, n_canon * es);
+  slab.add(&cd.split_row, total.splits);
+  slab.add(&cd.split_slot_ptr, total.splits ? total.splits + 1 : 0);
+  slab.add((uint8_t**)&cd.scratch, total.slots * std::max<int64_t>(N, 1) * acc_bytes);
+  if (csr_src) slab.add((uint8_t**)csr_src, n_canon * (wide ? 8 : 4));
+  TRY(slab.alloc(&cd.slab, bytes));
+  if (csr_src) p->vmap.csr_src_in_slab = true;
   row_emit_k<<<(unsigned)row_blocks, kThreads, 0, s>>>(rs, sums, total, cpos, ikey, ival, pre_row, pre_beg, pre_len,
                                                        cd.split_row, cd.split_slot_ptr);
   TRY(cudaGetLastError());
   TRY(radix_sort<int64_t>(&ikey, &ival, &ikey2, &ival2, n_it, 6, ar, s));
-  TRY(own(&cd.item_row, n_it, bytes));
-  TRY(own(&cd.item_ptr, n_it + 1, bytes));
   item_order_k<<<grid_for(n_it), kThreads, 0, s>>>(ival, n_it, pre_row, pre_len, cd.item_row, dlen);
   TRY(cudaGetLastError());
   TRY(excl_scan<int64_t>(dlen, cd.item_ptr, n_it, true, ar, s));
   cd.nnz = n_canon;  // the set's rows hold exactly its entries
-  const int es = dense_elem_bytes(p->dtype);
-  TRY(own(&cd.col, n_canon, bytes));
-  TRY(own((uint8_t**)&cd.val, n_canon * es, bytes));
-  if (csr_src && wide) TRY(own((int64_t**)csr_src, n_canon, p->vmap.bytes));
-  if (csr_src && !wide) TRY(own((int32_t**)csr_src, n_canon, p->vmap.bytes));
   if (n_canon) {
     const ItemGatherArgs ga{ival, n_it, pre_beg, cd.item_ptr, csrc, n_canon, n_canon, A.ci, A.vals, p->scale,
                             scale_f32(p->scale), (float)tiny, remap, cd.col, cd.val, csr_src ? *csr_src : nullptr,
                             wide ? 1 : 0, n_sub};
     TRY(dispatch_item_gather(p->dtype, A.vals_f32, ga, s));
-  }
-  if (total.slots) {
-    const int acc_bytes = p->dtype == LOOPS_F64 ? 8 : 4;
-    TRY(own((uint8_t**)&cd.scratch, total.slots * std::max<int64_t>(N, 1) * acc_bytes, bytes));
   }
   return LOOPS_OK;
 }
@@ -1045,8 +1086,8 @@ loops_status validate_csr_device(const DevCsrIn& A, loops_dtype dtype, cudaStrea
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(&h, d, sizeof(h), cudaMemcpyDeviceToHost, s);
-  cudaFreeAsync(d, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  cudaFreeAsync(d, s);  // after the synchronisation, at which the pool would unmap it
   TRY(e);
   // reported in the order the host validation checks them
   if (h.rp0 != 0) { set_error("row_ptr[0] != 0"); return LOOPS_ERR_INVALID_CSR; }
