@@ -74,20 +74,29 @@ __device__ __forceinline__ void ldsm_x2_trans(uint32_t addr, uint32_t& r0, uint3
                : "=r"(r0), "=r"(r1) : "r"(addr));
 }
 
-constexpr int kStages = 4;
+// One warp per work unit and CT = 8 * NF columns, kHmmaUnits independent warps per CTA. BULK: B rows
+// are fetched with cp.async.bulk (needs 16-byte aligned rows and a multiple-of-8 N); otherwise the
+// lanes copy them element-wise.
+//
+// Bound by the latency of a unit's chain (unit, columns, B rows, C): most units have a few groups, so
+// what counts is units in flight per SM. A warp of its own needs no CTA barrier and kStages = 2
+// stages let more of them in, all of a short unit's rows in flight at once. Block mix, N = 64,
+// BF16 (32,780 units of two groups), whole SpMM: 237 -> 197 us, against four warps on 16 columns each
+// with a barrier per group and four stages; three stages 218 us, N = 256 on 2^18 rows 178 -> 164 us.
+constexpr int kStages = 2;
+constexpr int kHmmaUnits = 2;
 
-// WARPS warps, each owning NF n8-fragments: the CTA covers CT = WARPS * 8 * NF columns of one
-// row block. BULK: B rows are fetched with cp.async.bulk (needs 16-byte aligned rows and a
-// multiple-of-8 N); otherwise the threads copy them element-wise.
-template <class T, int WARPS, int NF, bool BULK>
-__global__ void __launch_bounds__(WARPS * 32) bcsr_hmma(BcsrKArgs a) {
-  constexpr int CT = WARPS * 8 * NF;
+template <class T, int NF, bool BULK>
+__global__ void __launch_bounds__(kHmmaUnits * 32) bcsr_hmma(BcsrKArgs a) {
+  constexpr int CT = 8 * NF;
   constexpr int RS = CT + 8;  // smem row stride in elements (+16 B: conflict-free ldmatrix)
-  __shared__ __align__(128) T sB[kStages][16][RS];
-  __shared__ __align__(8) uint64_t bar[kStages];
-  const int tid = threadIdx.x;
-  const int warp = tid >> 5, lane = tid & 31;
-  const int64_t u = blockIdx.x;
+  __shared__ __align__(128) T sB_all[kHmmaUnits][kStages][16][RS];
+  __shared__ __align__(8) uint64_t bar_all[kHmmaUnits][kStages];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t u = (int64_t)blockIdx.x * kHmmaUnits + warp;
+  if (u >= a.n_units) return;  // a warp leaves as a whole; no barrier spans warps
+  T (*sB)[16][RS] = sB_all[warp];
+  uint64_t* bar = bar_all[warp];
   const int32_t b = a.unit_block[u];
   const int64_t rb = a.rb_id[b];
   const int64_t t0 = a.unit_t0[u];
@@ -99,37 +108,37 @@ __global__ void __launch_bounds__(WARPS * 32) bcsr_hmma(BcsrKArgs a) {
   const uint4* Af = reinterpret_cast<const uint4*>(a.tile_val) + (t0 / 16) * 32;
   const int32_t* cols = a.tile_col + t0;
 
-  if (BULK && tid == 0) {
-    for (int s = 0; s < kStages; ++s) mbar_init(&bar[s], 1);
-    fence_mbar_init();
+  if (BULK) {
+    if (lane == 0) {
+      for (int s = 0; s < kStages; ++s) mbar_init(&bar[s], 1);
+      fence_mbar_init();
+    }
+    __syncwarp();
   }
-  __syncthreads();
 
-  // stage g: B rows of tiles g*16 .. g*16+15 into sB[g % kStages]. With bulk copies, lane k
-  // of warp 0 (k < 16) fetches row k: a padding tile's row (column -1) is zero-filled by its
-  // lane first, then lane 0 announces the stage's total bytes on its barrier (its arrival
-  // releases the zero rows to the waiting threads), then the lanes issue their copies at once.
+  // stage g: B rows of tiles g*16 .. g*16+15 into sB[g % kStages]. With bulk copies, lane k (k < 16)
+  // fetches row k: a padding tile's row (column -1) is zero-filled by its lane first, then lane
+  // 0 announces the stage's total bytes on its barrier, then the lanes issue their copies at
+  // once. The caller has synchronised the warp since the stage was last read.
   auto issue = [&](int g) {
     const int s = g % kStages;
     if (BULK) {
-      if (warp == 0) {
-        const uint32_t row_bytes = (uint32_t)width * sizeof(T);
-        const int32_t c = lane < 16 ? cols[g * 16 + lane] : -1;
-        if (lane < 16 && c < 0) {
-          uint4* z = reinterpret_cast<uint4*>(&sB[s][lane][0]);
-          for (int q = 0; q < CT * (int)sizeof(T) / 16; ++q) z[q] = make_uint4(0, 0, 0, 0);
-        }
-        const uint32_t bytes = __reduce_add_sync(0xffffffffu, (lane < 16 && c >= 0) ? row_bytes : 0u);
-        __syncwarp();
-        if (lane == 0) mbar_arrive_expect_tx(&bar[s], bytes);
-        __syncwarp();
-        if (lane < 16 && c >= 0) {
-          fence_proxy_async_smem();
-          bulk_g2s(&sB[s][lane][0], Bp + (int64_t)c * a.ldb + n0, row_bytes, &bar[s]);
-        }
+      const uint32_t row_bytes = (uint32_t)width * sizeof(T);
+      const int32_t c = lane < 16 ? cols[g * 16 + lane] : -1;
+      if (lane < 16 && c < 0) {
+        uint4* z = reinterpret_cast<uint4*>(&sB[s][lane][0]);
+        for (int q = 0; q < CT * (int)sizeof(T) / 16; ++q) z[q] = make_uint4(0, 0, 0, 0);
+      }
+      const uint32_t bytes = __reduce_add_sync(0xffffffffu, (lane < 16 && c >= 0) ? row_bytes : 0u);
+      __syncwarp();
+      if (lane == 0) mbar_arrive_expect_tx(&bar[s], bytes);
+      __syncwarp();
+      if (lane < 16 && c >= 0) {
+        fence_proxy_async_smem();
+        bulk_g2s(&sB[s][lane][0], Bp + (int64_t)c * a.ldb + n0, row_bytes, &bar[s]);
       }
     } else {
-      for (int i = tid; i < 16 * CT; i += WARPS * 32) {
+      for (int i = lane; i < 16 * CT; i += 32) {
         const int k = i / CT, n = i % CT;
         const int32_t c = cols[g * 16 + k];
         sB[s][k][n] = (c >= 0 && n < width) ? Bp[(int64_t)c * a.ldb + n0 + n] : T(0.f);
@@ -143,28 +152,32 @@ __global__ void __launch_bounds__(WARPS * 32) bcsr_hmma(BcsrKArgs a) {
 #pragma unroll
     for (int i = 0; i < 4; ++i) acc[f][i] = 0.f;
 
-  bool failed = false;
-  int fail_g = -1;
-  const int pre = min(n_groups, kStages - 1);
-  for (int g = 0; g < pre; ++g) issue(g);
+  for (int g = 0; g < min(n_groups, kStages); ++g) issue(g);
   for (int g = 0; g < n_groups; ++g) {
-    // every warp is done with stage (g - 1) % kStages; a failed wait anywhere stops the CTA
-    if (__syncthreads_or(failed)) { fail_g = g - 1; break; }
-    if (g + kStages - 1 < n_groups) issue(g + kStages - 1);
-    if (!BULK) __syncthreads();
-    const int s = g % kStages;
-    if (BULK && !mbar_wait_bounded(&bar[s], (uint32_t)((g / kStages) & 1), a.max_polls)) {
-      failed = true;
-      atomicOr(a.err, kErrWaitTimeout);
-      continue;
-    }
     const uint4 af = __ldg(Af + (int64_t)g * 32 + lane);
+    const int s = g % kStages;
+    if (BULK) {
+      const bool ok = mbar_wait_bounded(&bar[s], (uint32_t)((g / kStages) & 1), a.max_polls);
+      if (__any_sync(0xffffffffu, !ok)) {
+        // a wait gave up: record it, let every copy that may still be in flight into this warp's
+        // shared memory land (bounded), then leave without the store
+        if (lane == 0) {
+          atomicOr(a.err, kErrWaitTimeout);
+          for (int h = g; h < min(n_groups, g + kStages); ++h)
+            mbar_wait_bounded(&bar[h % kStages], (uint32_t)((h / kStages) & 1), 1 << 20);
+        }
+        __syncwarp();
+        return;
+      }
+    } else {
+      __syncwarp();
+    }
     // lanes 0-7 / 8-15 / 16-23 / 24-31 address rows k of the four 8x8 matrices:
     // (k 0-7, frag f), (k 8-15, frag f), (k 0-7, frag f+1), (k 8-15, frag f+1)
     const int mi = lane >> 3, r = lane & 7;
 #pragma unroll
     for (int f = 0; f < NF; f += 2) {
-      const int ncol = (warp * NF + f) * 8;
+      const int ncol = f * 8;
       if (f + 1 < NF) {
         const uint32_t addr = smem_addr(&sB[s][r + 8 * (mi & 1)][ncol + 8 * (mi >> 1)]);
         uint32_t b0, b1, b2, b3;
@@ -178,17 +191,8 @@ __global__ void __launch_bounds__(WARPS * 32) bcsr_hmma(BcsrKArgs a) {
         mma16816<T>(acc[f], af, b0, b1);
       }
     }
-  }
-  if (__syncthreads_or(failed) && fail_g < 0) fail_g = n_groups - 1;
-  if (BULK && fail_g >= 0) {
-    // a wait gave up: before leaving, let every copy that may still be in flight into this
-    // CTA's shared memory land (bounded), then skip the store
-    if (tid == 0) {
-      const int last = min(n_groups - 1, fail_g + kStages - 1);
-      for (int g = fail_g; g <= last; ++g) mbar_wait_bounded(&bar[g % kStages], (uint32_t)((g / kStages) & 1), 1 << 20);
-    }
-    __syncthreads();
-    return;
+    __syncwarp();  // every lane has read the stage
+    if (g + kStages < n_groups) issue(g + kStages);
   }
   // epilogue: acc[f] = C rows (q, q + 8) x columns (2t, 2t + 1) of fragment f
   const int q = lane >> 2, t = lane & 3;
@@ -198,7 +202,7 @@ __global__ void __launch_bounds__(WARPS * 32) bcsr_hmma(BcsrKArgs a) {
     float* P = reinterpret_cast<float*>(a.scratch) + (int64_t)slot * 16 * a.N;
 #pragma unroll
     for (int f = 0; f < NF; ++f) {
-      const int64_t n = n0 + (warp * NF + f) * 8 + 2 * t;
+      const int64_t n = n0 + f * 8 + 2 * t;
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         float* pp = P + (int64_t)(q + 8 * h) * a.N + n;
@@ -210,7 +214,7 @@ __global__ void __launch_bounds__(WARPS * 32) bcsr_hmma(BcsrKArgs a) {
   }
 #pragma unroll
   for (int f = 0; f < NF; ++f) {
-    const int64_t n = n0 + (warp * NF + f) * 8 + 2 * t;
+    const int64_t n = n0 + f * 8 + 2 * t;
     float s0 = a.inv_scale_f, s1 = a.inv_scale_f;
     if (a.col_scale) {
       if (n < a.N) s0 *= a.col_scale[n];
@@ -232,26 +236,26 @@ __global__ void __launch_bounds__(WARPS * 32) bcsr_hmma(BcsrKArgs a) {
   }
 }
 
-template <class T, int WARPS, int NF>
+template <class T, int NF>
 cudaError_t launch_hmma_cfg(const BcsrKArgs& a, bool bulk, cudaStream_t s) {
-  constexpr int CT = WARPS * 8 * NF;
-  dim3 grid((unsigned)a.n_units, (unsigned)((a.N + CT - 1) / CT));
-  if (bulk) bcsr_hmma<T, WARPS, NF, true><<<grid, WARPS * 32, 0, s>>>(a);
-  else bcsr_hmma<T, WARPS, NF, false><<<grid, WARPS * 32, 0, s>>>(a);
+  constexpr int CT = 8 * NF;
+  dim3 grid((unsigned)((a.n_units + kHmmaUnits - 1) / kHmmaUnits), (unsigned)((a.N + CT - 1) / CT));
+  if (bulk) bcsr_hmma<T, NF, true><<<grid, kHmmaUnits * 32, 0, s>>>(a);
+  else bcsr_hmma<T, NF, false><<<grid, kHmmaUnits * 32, 0, s>>>(a);
   return cudaGetLastError();
 }
 
-// Column tile of a CTA: the plan's bcsr_ntile when the autotuner set it (32, 64 or 128), else
+// Column tile of a warp: the plan's bcsr_ntile when the autotuner set it (32, 64 or 128), else
 // the smallest of 8 .. 128 that covers N.
 template <class T>
 cudaError_t launch_hmma(const BcsrKArgs& a, int ntile, cudaStream_t s) {
   const bool bulk = (a.N % 8 == 0) && ((uintptr_t)a.B % 16 == 0) && ((a.ldb * 2) % 16 == 0);
   const int64_t ct = ntile > 0 ? ntile : (a.N <= 8 ? 8 : a.N <= 16 ? 16 : a.N <= 32 ? 32 : a.N <= 64 ? 64 : 128);
-  if (ct <= 8) return launch_hmma_cfg<T, 1, 1>(a, bulk, s);
-  if (ct <= 16) return launch_hmma_cfg<T, 1, 2>(a, bulk, s);
-  if (ct <= 32) return launch_hmma_cfg<T, 2, 2>(a, bulk, s);
-  if (ct <= 64) return launch_hmma_cfg<T, 4, 2>(a, bulk, s);
-  return launch_hmma_cfg<T, 4, 4>(a, bulk, s);
+  if (ct <= 8) return launch_hmma_cfg<T, 1>(a, bulk, s);
+  if (ct <= 16) return launch_hmma_cfg<T, 2>(a, bulk, s);
+  if (ct <= 32) return launch_hmma_cfg<T, 4>(a, bulk, s);
+  if (ct <= 64) return launch_hmma_cfg<T, 8>(a, bulk, s);
+  return launch_hmma_cfg<T, 16>(a, bulk, s);
 }
 
 // ------------------------------------------------------------------ F64: FP64 FMAs on the entries
