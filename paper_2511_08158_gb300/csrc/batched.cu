@@ -258,10 +258,10 @@ __global__ void __launch_bounds__(256, csr_min_blocks<Tr>()) batched_csr(const B
 // B_r 8 two tiles at 4 blocks beat four at 3 (batch of 128 matrices 755 -> 724 us, with the
 // unpredicated loads; N = 16, 32, 64 of the 512-matrix batch 119, 234, 352 -> 112, 222, 323 us) and
 // three at either; one tile, or two at 5 blocks, spill (1.4x the call). B_r 16 holds 64
-// accumulators per lane: two tiles at 2 blocks.
-constexpr int kFfmaTiles = 2;
+// accumulators per lane at 2 blocks: three tiles (batch of 128 matrices 762 us; two 809, one 825).
 template <int BR>
 struct FfmaShape {
+  static constexpr int kTiles = BR == 16 ? 3 : 2;
   static constexpr int kMinBlocks = BR == 16 ? 2 : 4;
 };
 
@@ -269,7 +269,7 @@ struct FfmaShape {
 // T tiles' B vectors and A values are loaded before their FMAs.
 template <int BR, int G, bool FULL>
 __device__ __forceinline__ void ffma_unit(const BatchDesc& d, int64_t u, int sub) {
-  constexpr int T = kFfmaTiles;
+  constexpr int T = FfmaShape<BR>::kTiles;
   const int32_t b = d.unit_block[u];
   const int64_t rb = d.rb_id[b];
   const int64_t t0 = d.unit_t0[u], t1 = d.unit_t1[u];
