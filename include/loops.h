@@ -76,7 +76,7 @@ typedef struct {
  *      performance model picks tau (see LOOPS_TAU_MODEL). Other tau < 0: autotune (time
  *      candidate thresholds on the plan's stream, the L2 flushed before each timed call;
  *      for F32 with block_rows 0 also B_r 8 and 16; then, on the chosen split, the CSR
- *      kernel's vectors per lane and the F16/BF16 BCSR kernel's columns per CTA -- reported
+ *      kernel's vectors per lane and the F16/BF16 BCSR kernel's columns per warp -- reported
  *      by loops_plan_info); +inf: CSR only (the pure vector-unit configuration of Sec. 4.3);
  *      0: every non-empty block BCSR (pure matrix unit).
  * block_rows: B_r (tile height); 0 = default (8 for F64, 16 otherwise; F32 autotuning tries
@@ -132,7 +132,7 @@ typedef struct {
                               3 contiguous split (paper mode) */
   int32_t csr_lane_vectors;/* CSR kernel: 16-byte column vectors per lane the autotuner chose
                               (1 or 2); 0: the built-in rule */
-  int32_t bcsr_col_tile;   /* F16/BF16 BCSR kernel: columns per CTA the autotuner chose (32, 64,
+  int32_t bcsr_col_tile;   /* F16/BF16 BCSR kernel: columns per warp the autotuner chose (32, 64,
                               128); 0: the smallest tile covering N */
   int32_t reserved0;
   double model_gflops;     /* tau_source 2: the Eq. 2 prediction for the chosen split; else NaN */

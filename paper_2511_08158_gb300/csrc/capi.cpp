@@ -468,7 +468,7 @@ cudaError_t L2Flush::run(cudaStream_t s) {
 // Autotuner: times C = A.B for candidate split thresholds (and, for F32, either tile height)
 // on synthetic B with the L2 flushed before each timed call, keeps the fastest, then times the
 // shapes of its kernels on that plan: the CSR kernel's 16-byte column vectors per lane (1 or
-// 2) and, for F16/BF16, the BCSR kernel's columns per CTA (32, 64 or 128). Candidates that give
+// 2) and, for F16/BF16, the BCSR kernel's columns per warp (32, 64 or 128). Candidates that give
 // the same row-block split as an earlier one are skipped.
 loops_status autotune_tau(const PlanBuilder& build, int64_t n_rows, int64_t n_cols, int64_t nnz, int64_t N,
                           loops_dtype dtype, int32_t split_len, bool try_tile_split, int32_t br, bool try_br,
