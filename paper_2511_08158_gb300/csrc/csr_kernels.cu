@@ -404,6 +404,27 @@ struct BwdKArgs {
   const float* b_scale;
 };
 
+// The dot products of an item's entries with the column weights on dC's side, for the rows j where a
+// non-zero element of B[j, :] times its weight leaves binary32's normal range: the loop of
+// csr_backward_vec would multiply a zero of dC by infinity there, or lose the element. Plain loops,
+// out of line: such weights are far from what a per-column scaling gives.
+template <class Tr, int G>
+__device__ __noinline__ void weighted_dots(const int32_t* col, const int32_t* src, int32_t len, int sub, unsigned gmask,
+                                           const typename Tr::TB* dC, int64_t lddc, const typename Tr::TB* Brow,
+                                           const float* dc_scale, const float* b_scale, int64_t N,
+                                           typename Tr::TC* dvals) {
+  for (int32_t k = 0; k < len; ++k) {
+    const typename Tr::TB* drow = dC + (int64_t)col[k] * lddc;
+    float s = 0.f;
+    for (int64_t n = sub; n < N; n += G) {
+      const float weight = (dc_scale ? dc_scale[n] : 1.f) * (b_scale ? b_scale[n] : 1.f);
+      s = fma(Tr::to_acc(drow[n]) * weight, Tr::to_acc(Brow[n]), s);
+    }
+    for (int off = G / 2; off > 0; off >>= 1) s += __shfl_xor_sync(gmask, s, off, G);
+    if (sub == 0) dvals[src[k]] = s;
+  }
+}
+
 template <class Tr, int G, int VPL, bool FULL>
 __global__ void __launch_bounds__(kCsrThreads, (BwdShape<Tr, VPL>::kWarps * 32 / kCsrThreads))
     csr_backward_vec(CsrKArgs a, BwdKArgs w) {
@@ -445,6 +466,7 @@ __global__ void __launch_bounds__(kCsrThreads, (BwdShape<Tr, VPL>::kWarps * 32 /
   const int32_t n0 = sub * VE;
   bool ok[VPL];
   TAcc acc[VPL][VE], bj[VPL][VE];
+  bool lossy = false;  // a non-zero element of B[j, :] leaves binary32's normal range with its weight
 #pragma unroll
   for (int p = 0; p < VPL; ++p) {
     const int32_t n = n0 + p * G * VE;
@@ -452,9 +474,19 @@ __global__ void __launch_bounds__(kCsrThreads, (BwdShape<Tr, VPL>::kWarps * 32 /
     unpack16<Tr>(ldg16_if(ok[p], reinterpret_cast<const TB*>(w.B) + (int64_t)j * w.ldb + n), bj[p]);
     if constexpr (Tr::kScaled) {
       if (ok[p]) {
+        float b[VE], lo = 1.f, hi = 0.f;
 #pragma unroll
-        for (int e = 0; e < VE; ++e)
+        for (int e = 0; e < VE; ++e) {
+          b[e] = bj[p][e];
           bj[p][e] *= (w.dc_scale ? w.dc_scale[n + e] : 1.f) * (w.b_scale ? w.b_scale[n + e] : 1.f);
+          lo = fminf(lo, fabsf(bj[p][e]));
+          hi = fmaxf(hi, fabsf(bj[p][e]));
+        }
+        lossy = lossy || hi > 0x1.fffffep127f;
+        if (lo < 0x1p-126f) {  // a zero of B, or an element that the product took there
+#pragma unroll
+          for (int e = 0; e < VE; ++e) lossy |= (b[e] != 0.f) & (fabsf(bj[p][e]) < 0x1p-126f);
+        }
       }
     }
 #pragma unroll
@@ -551,6 +583,11 @@ __global__ void __launch_bounds__(kCsrThreads, (BwdShape<Tr, VPL>::kWarps * 32 /
     }
   }
   store_item<Tr, G, VPL>(a, row, n0, ok, acc);
+  if constexpr (Tr::kScaled) {
+    if (__any_sync(gmask, lossy))  // also orders the stores above before those that replace them
+      weighted_dots<Tr, G>(a.col + beg, w.src + beg, len, sub, gmask, reinterpret_cast<const TB*>(a.B), a.ldb,
+                           reinterpret_cast<const TB*>(w.B) + (int64_t)j * w.ldb, w.dc_scale, w.b_scale, a.N, dvals);
+  }
 }
 
 inline int next_pow2(int64_t x) {
