@@ -18,6 +18,10 @@
  *    dimension (elements between consecutive rows), ld >= number of columns.
  *  - Every GPU call is ordered on the given stream (NULL = legacy default stream) and does
  *    not synchronise the device unless its comment says so.
+ *  - A plan with split rows or split BCSR blocks (CSR rows above 512 entries with the default
+ *    split_len: n_segments > 0; blocks above 256 tiles) keeps partial sums in its own device
+ *    memory during loops_spmm and loops_spmm_backward: such calls on one plan must not overlap
+ *    on the GPU. Calls on a plan without them may run on several streams at once.
  *  - Element types per plan dtype:
  *        dtype      A values stored   B, dC      C, dB, dvals   accumulation
  *        LOOPS_F64  f64               f64        f64            f64 (DFMA)
@@ -99,7 +103,8 @@ typedef struct {
   int32_t contiguous_split;
   int64_t r_boundary;
   int32_t want_backward;
-  int32_t split_len;      /* CSR rows longer than this are split in segments; 0 = default */
+  int32_t split_len;      /* CSR rows longer than this are split in segments of this length; 0 =
+                             default: rows above 512 entries, in segments of 64 to 512 by size */
   int32_t tile_min;
   int32_t reserved[5];
 } loops_plan_opts;

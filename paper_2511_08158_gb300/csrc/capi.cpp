@@ -217,13 +217,15 @@ void destroy_plan(loops_plan_s* p) {
   delete p;
 }
 
-// Longest CSR item where the caller gives no split_len. One lane group works through an item a few
-// entries at a time, so the longest item bounds a small problem's time (512 entries: 50 to 80 us),
-// while cutting costs partial sums. The length follows the entries per resident lane group (about
+// Entries that one lane group takes of a long CSR row where the caller gives no split_len: the length of
+// the segments of rows above kDefaultCutLen entries, and what the teams of shorter rows are sized by.
+// A group works through its entries a few at a time, so the longest chain bounds a small problem's
+// time (512 entries: 50 to 80 us). Only rows above kDefaultCutLen become segments: their partial
+// sums are the plan's memory, which calls on two streams would share. The length follows the entries per resident lane group (about
 // 2^18 lanes on the GPU; a group has the lanes of two 16-byte vectors each, 8 to 32), in [64, 512].
-// Measured against 512 for every size: graphs of 4,000 and 30,000 nodes (N = 64, 128, FP32) 69 -> 19
-// and 80 -> 24 us, 100,000 nodes (N = 64, BF16) 75 -> 31 us, 500,000 nodes (N = 128, FP16) 198 ->
-// 162 us; 64 for every size costs the GCN layer (N = 256, FP32) 7 %.
+// Measured against one group for every row of up to 512 entries: graphs of 4,000 and 30,000 nodes (N =
+// 64, 128, FP32) 80 -> 19 and 96 -> 23 us; with segments of 64 for every size the GCN layer (N = 256, FP32)
+// loses 7 %.
 static int32_t default_split_len(int64_t nnz, int64_t N, loops_dtype dtype) {
   const int64_t row_bytes = N * dense_elem_bytes(dtype);
   int64_t lanes = 8;
@@ -250,6 +252,8 @@ static loops_plan_s* new_plan(int64_t n_rows, int64_t n_cols, int64_t nnz, int64
   p->tau = tau;
   p->opts = o;
   p->split_len = o.split_len > 0 ? o.split_len : default_split_len(nnz, N, dtype);
+  p->cut_len = o.split_len > 0 ? o.split_len : kDefaultCutLen;
+  p->team_len = LOOPS_CSR_ITEMS_BY_LENGTH && p->split_len < p->cut_len ? p->split_len : 0;
   p->tile_min = o.tile_min > 1 ? o.tile_min : 0;
   p->transposed = nullptr;
   p->d_error = nullptr;

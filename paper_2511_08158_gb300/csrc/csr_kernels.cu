@@ -18,6 +18,24 @@ namespace loops {
 
 namespace {
 
+constexpr int kCsrThreads = 128;
+constexpr int32_t kPastEnd = 1 << 30;  // an entry past every item's end
+
+// The long rows of a team launch, in three classes (longest first) of one team size each. They are the
+// items after the segments of cut rows, and the classes have the first blocks, in order.
+constexpr int kTeamMax = 8;     // groups
+constexpr int kTeamChunk = 32;  // entries
+struct Teams {
+  int32_t n_slots;
+  int32_t n[3], log_size[3], block_end[3];
+};
+
+// Threads of a block: a team of any size fits.
+template <int G, bool TEAM>
+struct CsrBlock {
+  static constexpr int kThreads = TEAM && G * kTeamMax > kCsrThreads ? G * kTeamMax : kCsrThreads;
+};
+
 struct CsrKArgs {
   const int32_t* item_row;
   const int64_t* item_ptr;
@@ -35,6 +53,7 @@ struct CsrKArgs {
   double inv_scale_d;
   int64_t N;
   int accumulate;        // add to C (rows a BCSR part wrote first) instead of overwriting it
+  Teams team;            // team launches only
 };
 
 template <class Tr>
@@ -81,6 +100,74 @@ __device__ __forceinline__ void fetch_entries(const CsrKArgs& a, int64_t beg, in
       v[r] = Tr::load_v(reinterpret_cast<const TB*>(a.val) + beg + k);
     }
   }
+}
+
+// The item of a lane group and its part of the item's entries. One group has a whole item, or in a team
+// launch a long row has a team of groups that take kTeamChunk entries each in turn, whatever G, and
+// whose sums meet in team_sum in one order: a row's bits do not depend on the kernel or its shape.
+struct Share {
+  int64_t item;
+  int32_t first;     // entry
+  int32_t skip;      // entries that the other groups take between two of its pieces
+  int32_t log_size;  // of the team; -1: one group
+  bool live;
+};
+template <int G, bool TEAM>
+__device__ __forceinline__ Share share_of(const CsrKArgs& a) {
+  constexpr int kThreads = CsrBlock<G, TEAM>::kThreads;
+  if constexpr (TEAM) {
+    const Teams& t = a.team;
+    const int b = (int)blockIdx.x, group = (int)threadIdx.x / G;
+    if (b < t.block_end[2]) {
+      const int r = b < t.block_end[0] ? 0 : b < t.block_end[1] ? 1 : 2;
+      const int ls = t.log_size[r];
+      const int at = ((b - (r ? t.block_end[r - 1] : 0)) * (kThreads / G) + group) >> ls;
+      const bool live = at < t.n[r];  // the last block of a class may have teams without a row
+      const int before = (r > 0 ? t.n[0] : 0) + (r > 1 ? t.n[1] : 0);
+      return {(int64_t)t.n_slots + before + (live ? at : 0),
+              live ? (group & ((1 << ls) - 1)) * kTeamChunk : kPastEnd, ((1 << ls) - 1) * kTeamChunk, ls, live};
+    }
+    const int64_t g = (int64_t)(b - t.block_end[2]) * (kThreads / G) + group;
+    return {g < t.n_slots ? g : g + t.n[0] + t.n[1] + t.n[2], 0, 0, -1, true};
+  } else {
+    return {((int64_t)blockIdx.x * kThreads + threadIdx.x) / G, 0, 0, -1, true};
+  }
+}
+
+// First entry of the chunk after the one at k0.
+template <int CH, bool TEAM>
+__device__ __forceinline__ int32_t next_chunk(const Share& sh, int32_t k0) {
+  static_assert(kTeamChunk % CH == 0, "chunks tile a group's piece");
+  k0 += CH;
+  return TEAM && k0 % kTeamChunk == 0 ? k0 + sh.skip : k0;
+}
+
+// Sum of the accumulators over a team's groups, pairs first; true in the group that holds it. All
+// threads of the block are here (its teams have one size).
+template <int G, class TAcc, int P, int E>
+__device__ __forceinline__ bool team_sum(const Share& sh, TAcc (&acc)[P][E]) {
+  __shared__ TAcc part[CsrBlock<G, true>::kThreads / 32][P * E][G];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int lanes = G << sh.log_size;
+  __syncwarp();  // the groups' loops end apart
+#pragma unroll
+  for (int off = G; off < 32; off <<= 1) {
+    if (off >= lanes) break;
+#pragma unroll
+    for (int i = 0; i < P * E; ++i) acc[i / E][i % E] += __shfl_xor_sync(0xffffffffu, acc[i / E][i % E], off);
+  }
+  for (int h = 1; h < lanes / 32; h <<= 1) {  // a warp's sums are written once and read once
+    if (lane < G && (warp & (2 * h - 1)) == h) {
+#pragma unroll
+      for (int i = 0; i < P * E; ++i) part[warp][i][lane] = acc[i / E][i % E];
+    }
+    __syncthreads();
+    if (lane < G && (warp & (2 * h - 1)) == 0) {
+#pragma unroll
+      for (int i = 0; i < P * E; ++i) acc[i / E][i % E] += part[warp + h][i][lane];
+    }
+  }
+  return sh.live && ((int)threadIdx.x & (lanes - 1)) < G;
 }
 
 // Output of an item: its C row (scaled), or its slot of partial sums.
@@ -144,18 +231,17 @@ __device__ __forceinline__ void store_item(const CsrKArgs& a, int32_t row, int32
 //   the entries are read once per slice, and shorter pieces cost more instructions per byte.
 // FP64 is bound by the FP64 pipe: one entry at a time, so that no FMA is spent on a padded slot,
 // and no entries ahead; 48 warps per SM with one vector per lane (at 64 its 32 registers spill).
-constexpr int kCsrThreads = 128;
-
 template <class Tr, int VPL>
 struct CsrShape {
   static constexpr bool kF64 = std::is_same<Tr, TrF64>::value;
   static constexpr int kInFlight = kF64 ? 1 : (VPL == 1 ? 4 : 2);  // entries
   static constexpr bool kAhead = !kF64;  // load the next chunk's entries before this chunk's B rows
-  static constexpr int kMinBlocks = (kF64 && VPL == 1 ? 48 : 32) * 32 / kCsrThreads;
+  static constexpr int kWarps = kF64 && VPL == 1 ? 48 : 32;  // per SM
 };
 
-template <class Tr, int G, int VPL, bool FULL>
-__global__ void __launch_bounds__(kCsrThreads, (CsrShape<Tr, VPL>::kMinBlocks)) csr_spmm_vec(CsrKArgs a) {
+template <class Tr, int G, int VPL, bool FULL, bool TEAM>
+__global__ void __launch_bounds__((CsrBlock<G, TEAM>::kThreads), (CsrShape<Tr, VPL>::kWarps * 32 / CsrBlock<G, TEAM>::kThreads))
+    csr_spmm_vec(CsrKArgs a) {
   using TB = typename Tr::TB;
   using TAcc = typename Tr::TAcc;
   using TV = typename Tr::TV;
@@ -167,11 +253,12 @@ __global__ void __launch_bounds__(kCsrThreads, (CsrShape<Tr, VPL>::kMinBlocks)) 
   static_assert(CH % U == 0, "load batches tile the chunk");
   const int lane = threadIdx.x & 31;
   const int sub = lane & (G - 1);
-  const int64_t item = ((int64_t)blockIdx.x * kCsrThreads + threadIdx.x) / G;
+  const Share sh = share_of<G, TEAM>(a);
+  const int64_t item = sh.item;
   if (item >= a.n_items) return;  // a group leaves as a whole
   const unsigned gmask = (G == 32) ? 0xffffffffu : (((1u << G) - 1u) << (lane & ~(G - 1)));
   const int64_t beg = a.item_ptr[item];
-  const int32_t len = (int32_t)(a.item_ptr[item + 1] - beg);  // at most split_len
+  const int32_t len = (int32_t)(a.item_ptr[item + 1] - beg);  // a row that is not cut, or a segment
   const int32_t row = a.item_row[item];
   const int32_t n0 = (int32_t)blockIdx.y * (G * VPL * VE) + sub * VE;  // vector p starts at column n0 + p * G * VE
   bool ok[VPL];
@@ -186,15 +273,16 @@ __global__ void __launch_bounds__(kCsrThreads, (CsrShape<Tr, VPL>::kMinBlocks)) 
   const char* __restrict__ bl = reinterpret_cast<const char*>(a.B) + (int64_t)n0 * sizeof(TB);
   int32_t c[R], c_next[R];
   TV v[R], v_next[R];
-  if (AHEAD) fetch_entries<Tr, G>(a, beg, len, 0, sub, c_next, v_next);
-  for (int32_t k0 = 0; k0 < len; k0 += CH) {
+  if (AHEAD) fetch_entries<Tr, G>(a, beg, len, sh.first, sub, c_next, v_next);
+  for (int32_t k0 = sh.first, k1; k0 < len; k0 = k1) {
+    k1 = next_chunk<CH, TEAM>(sh, k0);
     if (AHEAD) {
 #pragma unroll
       for (int r = 0; r < R; ++r) {
         c[r] = c_next[r];
         v[r] = v_next[r];
       }
-      fetch_entries<Tr, G>(a, beg, len, k0 + CH, sub, c_next, v_next);
+      fetch_entries<Tr, G>(a, beg, len, k1, sub, c_next, v_next);
     } else {
       fetch_entries<Tr, G>(a, beg, len, k0, sub, c, v);
     }
@@ -234,6 +322,9 @@ __global__ void __launch_bounds__(kCsrThreads, (CsrShape<Tr, VPL>::kMinBlocks)) 
       }
     }
   }
+  if constexpr (TEAM) {
+    if (sh.log_size >= 0 && !team_sum<G>(sh, acc)) return;
+  }
   store_item<Tr, G, VPL>(a, row, n0, ok, acc);
 }
 
@@ -248,6 +339,9 @@ __global__ void __launch_bounds__(kCsrThreads, (CsrShape<Tr, VPL>::kMinBlocks)) 
 template <int CP, int VW>
 struct OddShape {
   static constexpr int kInFlight = CP * VW <= 2 ? 8 : (CP * VW <= 6 ? 4 : 2);  // entries
+  // Warps per SM that team launches must allow (0: as the compiler has it): the other instances reach
+  // them by themselves. FP32, N = 97 at 64 registers instead of 56: 14 % slower.
+  static constexpr int kTeamWarps = CP == 8 && VW == 1 ? 36 : CP == 6 && VW == 2 ? 32 : 0;
 };
 
 // VW adjacent elements of a row of B, zeros when off
@@ -267,8 +361,10 @@ __device__ __forceinline__ void load_piece(bool on, const TB* p, TB (&x)[VW]) {
   }
 }
 
-template <class Tr, int G, int CP, int VW>
-__global__ void __launch_bounds__(kCsrThreads) csr_spmm_odd(CsrKArgs a) {
+template <class Tr, int G, int CP, int VW, bool TEAM>
+__global__ void __launch_bounds__((CsrBlock<G, TEAM>::kThreads),
+                                  (TEAM && sizeof(typename Tr::TB) <= 4
+                                       ? OddShape<CP, VW>::kTeamWarps * 32 / CsrBlock<G, TEAM>::kThreads : 0)) csr_spmm_odd(CsrKArgs a) {
   using TB = typename Tr::TB;
   using TAcc = typename Tr::TAcc;
   using TC = typename Tr::TC;
@@ -277,7 +373,8 @@ __global__ void __launch_bounds__(kCsrThreads) csr_spmm_odd(CsrKArgs a) {
   static_assert(G % U == 0, "load batches tile the chunk of G entries");
   const int lane = threadIdx.x & 31;
   const int sub = lane & (G - 1);
-  const int64_t item = ((int64_t)blockIdx.x * kCsrThreads + threadIdx.x) / G;
+  const Share sh = share_of<G, TEAM>(a);
+  const int64_t item = sh.item;
   if (item >= a.n_items) return;  // a group leaves as a whole
   const unsigned gmask = (G == 32) ? 0xffffffffu : (((1u << G) - 1u) << (lane & ~(G - 1)));
   const int64_t beg = a.item_ptr[item];
@@ -295,11 +392,12 @@ __global__ void __launch_bounds__(kCsrThreads) csr_spmm_odd(CsrKArgs a) {
     for (int w = 0; w < VW; ++w) acc[i][w] = TAcc(0);
   int32_t c[1], c_next[1];
   TV v[1], v_next[1];
-  fetch_entries<Tr, G>(a, beg, len, 0, sub, c_next, v_next);
-  for (int32_t k0 = 0; k0 < len; k0 += G) {
+  fetch_entries<Tr, G>(a, beg, len, sh.first, sub, c_next, v_next);
+  for (int32_t k0 = sh.first, k1; k0 < len; k0 = k1) {
+    k1 = next_chunk<G, TEAM>(sh, k0);
     c[0] = c_next[0];
     v[0] = v_next[0];
-    fetch_entries<Tr, G>(a, beg, len, k0 + G, sub, c_next, v_next);
+    fetch_entries<Tr, G>(a, beg, len, k1, sub, c_next, v_next);
     const int cnt = min(len - k0, G);  // uniform in the group
     // entries past the chunk's end load nothing and carry zero values
     auto batch = [&](int e0, auto tail_tag) {
@@ -324,6 +422,9 @@ __global__ void __launch_bounds__(kCsrThreads) csr_spmm_odd(CsrKArgs a) {
     int e0 = 0;
     for (; e0 + U <= cnt; e0 += U) batch(e0, std::false_type());
     if (e0 < cnt) batch(e0, std::true_type());
+  }
+  if constexpr (TEAM) {
+    if (sh.log_size >= 0 && !team_sum<G>(sh, acc)) return;
   }
 #pragma unroll
   for (int i = 0; i < CP; ++i) {
@@ -408,12 +509,12 @@ struct BwdKArgs {
 // non-zero element of B[j, :] times its weight leaves binary32's normal range: the loop of
 // csr_backward_vec would multiply a zero of dC by infinity there, or lose the element. Plain loops,
 // out of line: such weights are far from what a per-column scaling gives.
-template <class Tr, int G>
-__device__ __noinline__ void weighted_dots(const int32_t* col, const int32_t* src, int32_t len, int sub, unsigned gmask,
-                                           const typename Tr::TB* dC, int64_t lddc, const typename Tr::TB* Brow,
-                                           const float* dc_scale, const float* b_scale, int64_t N,
-                                           typename Tr::TC* dvals) {
-  for (int32_t k = 0; k < len; ++k) {
+template <class Tr, int G, bool TEAM>
+__device__ __noinline__ void weighted_dots(const int32_t* col, const int32_t* src, int32_t len, const Share sh, int sub,
+                                           unsigned gmask, const typename Tr::TB* dC, int64_t lddc,
+                                           const typename Tr::TB* Brow, const float* dc_scale, const float* b_scale,
+                                           int64_t N, typename Tr::TC* dvals) {
+  for (int32_t k = sh.first; k < len; k = next_chunk<1, TEAM>(sh, k)) {
     const typename Tr::TB* drow = dC + (int64_t)col[k] * lddc;
     float s = 0.f;
     for (int64_t n = sub; n < N; n += G) {
@@ -425,8 +526,8 @@ __device__ __noinline__ void weighted_dots(const int32_t* col, const int32_t* sr
   }
 }
 
-template <class Tr, int G, int VPL, bool FULL>
-__global__ void __launch_bounds__(kCsrThreads, (BwdShape<Tr, VPL>::kWarps * 32 / kCsrThreads))
+template <class Tr, int G, int VPL, bool FULL, bool TEAM>
+__global__ void __launch_bounds__((CsrBlock<G, TEAM>::kThreads), (BwdShape<Tr, VPL>::kWarps * 32 / CsrBlock<G, TEAM>::kThreads))
     csr_backward_vec(CsrKArgs a, BwdKArgs w) {
   using TB = typename Tr::TB;
   using TAcc = typename Tr::TAcc;
@@ -439,7 +540,8 @@ __global__ void __launch_bounds__(kCsrThreads, (BwdShape<Tr, VPL>::kWarps * 32 /
   static_assert(CH % U == 0, "load batches tile the chunk");
   const int lane = threadIdx.x & 31;
   const int sub = lane & (G - 1);
-  const int64_t item = ((int64_t)blockIdx.x * kCsrThreads + threadIdx.x) / G;
+  const Share sh = share_of<G, TEAM>(a);
+  const int64_t item = sh.item;
   if (item >= a.n_items) return;  // a group leaves as a whole
   const unsigned gmask = (G == 32) ? 0xffffffffu : (((1u << G) - 1u) << (lane & ~(G - 1)));
   const int64_t beg = a.item_ptr[item];
@@ -452,7 +554,7 @@ __global__ void __launch_bounds__(kCsrThreads, (BwdShape<Tr, VPL>::kWarps * 32 /
   };
   int32_t c_next[R], x_next[R];
   TV v_next[R];
-  fetch(0, c_next, v_next, x_next);
+  fetch(sh.first, c_next, v_next, x_next);
   int32_t j = row;
   if (row < 0) {  // a segment: the split row that holds its slot
     const int32_t slot = -1 - row;
@@ -494,7 +596,8 @@ __global__ void __launch_bounds__(kCsrThreads, (BwdShape<Tr, VPL>::kWarps * 32 /
   }
   const char* __restrict__ dl = reinterpret_cast<const char*>(a.B) + (int64_t)n0 * sizeof(TB);
   TC* __restrict__ dvals = reinterpret_cast<TC*>(w.dvals);
-  for (int32_t k0 = 0; k0 < len; k0 += CH) {
+  for (int32_t k0 = sh.first, k1; k0 < len; k0 = k1) {
+    k1 = next_chunk<CH, TEAM>(sh, k0);
     int32_t c[R], x[R];
     TV v[R];
 #pragma unroll
@@ -503,7 +606,7 @@ __global__ void __launch_bounds__(kCsrThreads, (BwdShape<Tr, VPL>::kWarps * 32 /
       v[r] = v_next[r];
       x[r] = x_next[r];
     }
-    fetch(k0 + CH, c_next, v_next, x_next);
+    fetch(k1, c_next, v_next, x_next);
     const int cnt = min(len - k0, CH);  // uniform in the group
     // entries e0 .. e0 + U - 1 of the chunk; TAIL: those past its end load nothing, carry zero
     // values and are not stored
@@ -582,12 +685,16 @@ __global__ void __launch_bounds__(kCsrThreads, (BwdShape<Tr, VPL>::kWarps * 32 /
       }
     }
   }
-  store_item<Tr, G, VPL>(a, row, n0, ok, acc);
   if constexpr (Tr::kScaled) {
     if (__any_sync(gmask, lossy))  // also orders the stores above before those that replace them
-      weighted_dots<Tr, G>(a.col + beg, w.src + beg, len, sub, gmask, reinterpret_cast<const TB*>(a.B), a.ldb,
-                           reinterpret_cast<const TB*>(w.B) + (int64_t)j * w.ldb, w.dc_scale, w.b_scale, a.N, dvals);
+      weighted_dots<Tr, G, TEAM>(a.col + beg, w.src + beg, len, sh, sub, gmask, reinterpret_cast<const TB*>(a.B), a.ldb,
+                                 reinterpret_cast<const TB*>(w.B) + (int64_t)j * w.ldb, w.dc_scale, w.b_scale, a.N,
+                                 dvals);
   }
+  if constexpr (TEAM) {
+    if (sh.log_size >= 0 && !team_sum<G>(sh, acc)) return;
+  }
+  store_item<Tr, G, VPL>(a, row, n0, ok, acc);
 }
 
 inline int next_pow2(int64_t x) {
@@ -596,25 +703,50 @@ inline int next_pow2(int64_t x) {
   return p;
 }
 
-template <class Tr, int G, int VPL>
-cudaError_t launch_vec_g(const CsrKArgs& a, cudaStream_t s) {
-  constexpr int64_t per_chunk = (int64_t)G * VPL * Tr::kVE;
-  const dim3 grid((unsigned)((a.n_items * G + kCsrThreads - 1) / kCsrThreads),
-                  (unsigned)((a.N + per_chunk - 1) / per_chunk));
-  if (a.N % per_chunk == 0) csr_spmm_vec<Tr, G, VPL, true><<<grid, kCsrThreads, 0, s>>>(a);
-  else csr_spmm_vec<Tr, G, VPL, false><<<grid, kCsrThreads, 0, s>>>(a);
+// Launches one of the three item kernels (`kernel` takes whether there are teams) over its items and
+// `chunks` column chunks.
+template <int G, class K>
+cudaError_t launch_items(CsrKArgs a, const CsrDev& d, int64_t chunks, K kernel) {
+  const int64_t team_rows = d.n_long[0] + d.n_long[1] + d.n_long[2];
+  auto blocks_of = [](int64_t groups, int threads) { return (groups * G + threads - 1) / threads; };
+  if (team_rows == 0) {
+    constexpr int T = CsrBlock<G, false>::kThreads;
+    kernel(a, dim3((unsigned)blocks_of(a.n_items, T), (unsigned)chunks), T, std::false_type());
+    return cudaGetLastError();
+  }
+  constexpr int T = CsrBlock<G, true>::kThreads;
+  Teams& t = a.team;
+  t.n_slots = (int32_t)d.n_slots;
+  int64_t blocks = 0;
+  for (int r = 0; r < 3; ++r) {
+    t.n[r] = (int32_t)d.n_long[r];
+    t.log_size[r] = long_class_log_team(r, d.team_len);
+    blocks += blocks_of(d.n_long[r] << t.log_size[r], T);
+    t.block_end[r] = (int32_t)blocks;
+  }
+  blocks += blocks_of(a.n_items - team_rows, T);
+  kernel(a, dim3((unsigned)blocks, (unsigned)chunks), T, std::true_type());
   return cudaGetLastError();
 }
 
+template <class Tr, int G, int VPL>
+cudaError_t launch_vec_g(const CsrKArgs& a, const CsrDev& d, cudaStream_t s) {
+  constexpr int64_t per_chunk = (int64_t)G * VPL * Tr::kVE;
+  return launch_items<G>(a, d, (a.N + per_chunk - 1) / per_chunk, [&](const CsrKArgs& k, dim3 grid, int threads, auto team) {
+    constexpr bool T = decltype(team)::value;
+    if (k.N % per_chunk == 0) csr_spmm_vec<Tr, G, VPL, true, T><<<grid, threads, 0, s>>>(k);
+    else csr_spmm_vec<Tr, G, VPL, false, T><<<grid, threads, 0, s>>>(k);
+  });
+}
+
 template <class Tr, int VW>
-cudaError_t launch_odd_vw(const CsrKArgs& a, cudaStream_t s) {
+cudaError_t launch_odd_vw(const CsrKArgs& a, const CsrDev& d, cudaStream_t s) {
   const int64_t pieces = a.N / VW;
   auto go = [&](auto g_tag, auto cp_tag) {
     constexpr int G = decltype(g_tag)::value, CP = decltype(cp_tag)::value;
-    const dim3 grid((unsigned)((a.n_items * G + kCsrThreads - 1) / kCsrThreads),
-                    (unsigned)((pieces + G * CP - 1) / (G * CP)));
-    csr_spmm_odd<Tr, G, CP, VW><<<grid, kCsrThreads, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_items<G>(a, d, (pieces + G * CP - 1) / (G * CP), [&](const CsrKArgs& k, dim3 grid, int threads, auto team) {
+      csr_spmm_odd<Tr, G, CP, VW, decltype(team)::value><<<grid, threads, 0, s>>>(k);
+    });
   };
   using std::integral_constant;
   using G8 = integral_constant<int, 8>;
@@ -631,12 +763,12 @@ cudaError_t launch_odd_vw(const CsrKArgs& a, cudaStream_t s) {
 
 // Two columns per load where they divide N and every row of B keeps the load aligned.
 template <class Tr>
-cudaError_t launch_odd(const CsrKArgs& a, cudaStream_t s) {
+cudaError_t launch_odd(const CsrKArgs& a, const CsrDev& d, cudaStream_t s) {
   constexpr int64_t eb = sizeof(typename Tr::TB);
   if constexpr (eb <= 4) {
-    if (a.N % 2 == 0 && a.ldb % 2 == 0 && (uintptr_t)a.B % (2 * eb) == 0) return launch_odd_vw<Tr, 2>(a, s);
+    if (a.N % 2 == 0 && a.ldb % 2 == 0 && (uintptr_t)a.B % (2 * eb) == 0) return launch_odd_vw<Tr, 2>(a, d, s);
   }
-  return launch_odd_vw<Tr, 1>(a, s);
+  return launch_odd_vw<Tr, 1>(a, d, s);
 }
 
 CsrKArgs csr_args(const loops_plan_s* p, const CsrDev& d, const DenseArgs& da, bool accumulate) {
@@ -657,6 +789,7 @@ CsrKArgs csr_args(const loops_plan_s* p, const CsrDev& d, const DenseArgs& da, b
   a.inv_scale_f = da.inv_scale_f;
   a.inv_scale_d = da.inv_scale_d;
   a.N = da.N;
+  a.team = Teams();
   return a;
 }
 
@@ -692,15 +825,15 @@ cudaError_t launch_csr_t(const loops_plan_s* p, const CsrDev& d, const DenseArgs
       const int G = next_pow2(nv);
       const bool two = lv || nvec > 32;
       switch (G) {
-        case 1: e = two ? launch_vec_g<Tr, 1, 2>(a, s) : launch_vec_g<Tr, 1, 1>(a, s); break;
-        case 2: e = two ? launch_vec_g<Tr, 2, 2>(a, s) : launch_vec_g<Tr, 2, 1>(a, s); break;
-        case 4: e = two ? launch_vec_g<Tr, 4, 2>(a, s) : launch_vec_g<Tr, 4, 1>(a, s); break;
-        case 8: e = two ? launch_vec_g<Tr, 8, 2>(a, s) : launch_vec_g<Tr, 8, 1>(a, s); break;
-        case 16: e = two ? launch_vec_g<Tr, 16, 2>(a, s) : launch_vec_g<Tr, 16, 1>(a, s); break;
-        default: e = two ? launch_vec_g<Tr, 32, 2>(a, s) : launch_vec_g<Tr, 32, 1>(a, s); break;
+        case 1: e = two ? launch_vec_g<Tr, 1, 2>(a, d, s) : launch_vec_g<Tr, 1, 1>(a, d, s); break;
+        case 2: e = two ? launch_vec_g<Tr, 2, 2>(a, d, s) : launch_vec_g<Tr, 2, 1>(a, d, s); break;
+        case 4: e = two ? launch_vec_g<Tr, 4, 2>(a, d, s) : launch_vec_g<Tr, 4, 1>(a, d, s); break;
+        case 8: e = two ? launch_vec_g<Tr, 8, 2>(a, d, s) : launch_vec_g<Tr, 8, 1>(a, d, s); break;
+        case 16: e = two ? launch_vec_g<Tr, 16, 2>(a, d, s) : launch_vec_g<Tr, 16, 1>(a, d, s); break;
+        default: e = two ? launch_vec_g<Tr, 32, 2>(a, d, s) : launch_vec_g<Tr, 32, 1>(a, d, s); break;
       }
     } else {
-      e = launch_odd<Tr>(a, s);
+      e = launch_odd<Tr>(a, d, s);
     }
   }
   if (e == cudaSuccess) e = launch_split_reduce<Tr>(d, a, s);
@@ -713,10 +846,11 @@ cudaError_t launch_csr_backward_t(const CsrDev& d, const CsrKArgs& a, const BwdK
   auto go = [&](auto g_tag, auto p_tag) {
     constexpr int G = decltype(g_tag)::value;
     constexpr int VPL = decltype(p_tag)::value;
-    const unsigned blocks = (unsigned)((a.n_items * G + kCsrThreads - 1) / kCsrThreads);
-    if (a.N % (G * VPL * Tr::kVE) == 0) csr_backward_vec<Tr, G, VPL, true><<<blocks, kCsrThreads, 0, s>>>(a, w);
-    else csr_backward_vec<Tr, G, VPL, false><<<blocks, kCsrThreads, 0, s>>>(a, w);
-    return cudaGetLastError();
+    return launch_items<G>(a, d, 1, [&](const CsrKArgs& k, dim3 grid, int threads, auto team) {
+      constexpr bool T = decltype(team)::value;
+      if (!T && k.N % (G * VPL * Tr::kVE) == 0) csr_backward_vec<Tr, G, VPL, !T, T><<<grid, threads, 0, s>>>(k, w);
+      else csr_backward_vec<Tr, G, VPL, false, T><<<grid, threads, 0, s>>>(k, w);
+    });
   };
   using One = std::integral_constant<int, 1>;
   using Two = std::integral_constant<int, 2>;

@@ -1,9 +1,10 @@
 // Device layout of a plan's two parts, and its inverse (export back to canonical order).
 //
-// CSR part: rows become work items processed in storage order; rows longer than split_len
-// are cut into segments whose partial sums go to scratch slots and are summed afterwards in
+// CSR part: rows become work items processed in storage order; rows longer than cut_len
+// are cut into segments of split_len entries whose partial sums go to scratch slots and are summed afterwards in
 // slot order (deterministic). Items are ordered by decreasing length class, so the longest
-// work starts first; within a class the row order is kept.
+// work starts first (and the rows that a team may share follow the segments); within a class the
+// row order is kept.
 //
 // BCSR part: tile values are stored in the register-fragment order of the dtype's MMA, so a
 // lane loads its whole A fragment of a K-group with one vector load:
@@ -86,6 +87,26 @@ int bucket_of(int64_t len) {
 
 }  // namespace
 
+int64_t row_lanes(int64_t N, loops_dtype dtype) {
+  int64_t lanes = 8;
+  while (lanes * 32 < N * dense_elem_bytes(dtype)) lanes *= 2;
+  return lanes;
+}
+
+// Teams pay where the long rows at one group each would fill less than the lanes resident at once
+// (152 SMs of 32 warps, about 2^17): there the longest row bounds the time. More rows fill the chip,
+// and a team's start and sum only add to it. 30,000-node graph, 0.4 M entries, N = 128, FP32 (rows of up to
+// 512 entries): 96 us with one group per row, 23 with teams, 24 with the rows cut into segments; 20,000
+// rows of 100 entries, N = 128, BF16: 31 us with one group per row, 69 with every row cut in two. A class
+// that does not fit keeps the shorter ones out.
+void limit_teams(CsrDev& d, int64_t N, loops_dtype dtype) {
+  int64_t rows = 0;
+  for (int64_t& n : d.n_long) {
+    rows += n;
+    if (rows >= (1 << 17) / row_lanes(N, dtype)) n = 0;
+  }
+}
+
 loops_status upload_part(loops_plan_s* p, int64_t N) {
   const Canon& c = p->canon;
   PartDev& d = p->dev;
@@ -109,6 +130,8 @@ loops_status upload_part(loops_plan_s* p, int64_t N) {
     std::vector<It> items;
     const int64_t n_csr = (int64_t)c.csr_rows.size();
     const int64_t L = std::max<int64_t>(p->split_len, 1);
+    const int team_base = p->team_len > 0 ? bucket_of(p->team_len - 1) : -1;
+    cd.team_len = p->team_len;
     int64_t n_slots = 0;
     for (int64_t x = 0; x < n_csr; ++x) {
       const int32_t row = c.csr_rows[(size_t)x];
@@ -116,7 +139,7 @@ loops_status upload_part(loops_plan_s* p, int64_t N) {
       if (mixed != which) continue;
       const int64_t b = c.csr_ptr[(size_t)x], e = c.csr_ptr[(size_t)x + 1];
       const int64_t len = e - b;
-      if (len > L) {
+      if (len > p->cut_len) {
         cd.h_split_row.push_back(row);
         cd.h_split_slot_ptr.push_back((int32_t)n_slots);
         for (int64_t s0 = b; s0 < e; s0 += L) {
@@ -125,6 +148,8 @@ loops_status upload_part(loops_plan_s* p, int64_t N) {
         }
       } else {
         items.push_back({row, b, e, bucket_of(len)});
+        const int cls = long_class(items.back().bucket, team_base);
+        if (cls >= 0) ++cd.n_long[cls];
       }
     }
     cd.h_split_slot_ptr.push_back((int32_t)n_slots);
@@ -151,6 +176,7 @@ loops_status upload_part(loops_plan_s* p, int64_t N) {
       }
       cd.h_item_ptr[i + 1] = pos;
     }
+    limit_teams(cd, N, p->dtype);
     if (items.empty()) continue;
     encode_values(val.data(), val.size(), p->dtype, enc);
     if ((st = dev_upload(&cd.item_row, cd.h_item_row.data(), items.size(), bytes))) return st;

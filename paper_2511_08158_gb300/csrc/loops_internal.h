@@ -145,6 +145,10 @@ struct CsrDev {
   int32_t* split_row = nullptr;        // global C row of each split row
   int32_t* split_slot_ptr = nullptr;   // size n_split + 1
   void* scratch = nullptr;             // n_slots x N partial sums (accumulator type)
+  // uncut rows that a team of lane groups each takes, by class (long_class): the items after the
+  // segments, longest class first
+  int64_t n_long[3] = {0, 0, 0};
+  int32_t team_len = 0;
   void* slab = nullptr;                // when set, the one allocation that holds the arrays above
   // host mirrors used for export
   std::vector<int32_t> h_item_row;
@@ -165,6 +169,23 @@ constexpr int64_t kBcsrSplitTiles = 256;
 #ifndef LOOPS_CSR_ITEMS_BY_LENGTH
 #define LOOPS_CSR_ITEMS_BY_LENGTH 1
 #endif
+
+// Long CSR rows: class of CsrDev::n_long of a row in length class `bucket` (floor(log2(length + 1)), so
+// class r holds 2^(8 - r) - 1 to about 2^(9 - r) entries) with teams from class `base` on; -1: none.
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+inline int long_class(int bucket, int base) { return base < 6 || bucket < base ? -1 : bucket >= 8 ? 0 : 8 - bucket; }
+// log2 of the lane groups in a team: about the row's length / team_len
+inline int long_class_log_team(int r, int32_t team_len) {
+  int log = 0;
+  while (team_len > 0 && (team_len << log) < (512 >> r)) ++log;
+  return log;
+}
+
+// CSR rows longer than this are cut where the caller gives no split_len.
+constexpr int32_t kDefaultCutLen = 512;
+
 struct BcsrDev {
   int64_t n_rb = 0, n_tiles = 0;
   int32_t* rb_id = nullptr;
@@ -314,7 +335,9 @@ struct loops_plan_s {
   int32_t br, kpad;
   double tau;
   double scale;
-  int32_t split_len;
+  int32_t split_len;                   // length of the segments of a cut row (and of the SDDMM items)
+  int32_t cut_len;                     // rows longer than this are cut
+  int32_t team_len;                    // uncut rows of about this length or more may have a team; 0: none
   int32_t tile_min;                    // tile-level split threshold in effect (0: off)
   loops_plan_opts opts;
   loops::Canon canon;                  // host copy (canonical order)
@@ -357,6 +380,10 @@ void register_plan(const loops_plan_s* p);
 void unregister_plan(const loops_plan_s* p);
 
 // Device upload of a canonical partition (partition.cpp). Sets plan->dev.
+// Lane groups' lanes that a row of N columns takes: two 16-byte vectors per lane, at least 8.
+int64_t row_lanes(int64_t N, loops_dtype dtype);
+// Keeps the teams of d's long rows only where they pay (d.n_long, d.team_len are set).
+void limit_teams(CsrDev& d, int64_t N, loops_dtype dtype);
 loops_status upload_part(loops_plan_s* plan, int64_t N);
 void free_part(PartDev& d);
 // Build and upload the value maps; `remap` (optional) maps the plan's entry order to the

@@ -682,15 +682,16 @@ __device__ __forceinline__ int bucket_of_len(int64_t len) {  // floor(log2(len +
 }
 
 // Rows of one CSR set: set 0 takes every row of a CSR block (empty rows too; every row when
-// is_bcsr is null), set 1 the rows of BCSR blocks that have moved entries. Rows longer than L
-// become split rows of ceil(len / L) segments.
+// is_bcsr is null), set 1 the rows of BCSR blocks that have moved entries. Rows longer than `cut`
+// become split rows of ceil(len / L) segments; the uncut rows that a team may share are
+// counted by class (they follow the segments in the item order).
 struct RowSet {
   const int64_t* rp;
   const uint8_t* is_bcsr;
   const int32_t* rowlen1;
-  int64_t n_rows, L;
+  int64_t n_rows, L, cut;
   int32_t br;
-  int which;
+  int which, team_base;
   __device__ __forceinline__ int64_t len(int64_t i) const {  // -1: not in the set
     const bool in_b = is_bcsr && is_bcsr[i / br] != 0;
     if (which == 0) return in_b ? -1 : rp[i + 1] - rp[i];
@@ -698,45 +699,58 @@ struct RowSet {
   }
 };
 
-// Work items, partial-sum slots and split rows, of a row or summed.
+// Work items, partial-sum slots, split rows and long uncut rows, of a row or summed.
 struct RowCount {
-  int64_t items, slots, splits;
-  __device__ __forceinline__ void add(int64_t len, int64_t L) {
-    const int64_t segs = len > L ? (len + L - 1) / L : 0;
+  int64_t items, slots, splits, longs[3];
+  __device__ __forceinline__ void add(int64_t len, const RowSet& rs) {
+    const int64_t segs = len > rs.cut ? (len + rs.L - 1) / rs.L : 0;
     items += len < 0 ? 0 : (segs ? segs : 1);
     slots += segs;
     splits += segs > 0;
+    if (len < 0 || segs) return;
+    const int cls = long_class(bucket_of_len(len), rs.team_base);
+#pragma unroll
+    for (int r = 0; r < 3; ++r) longs[r] += cls == r;
   }
 };
 
-// The items are numbered by one scan of all three counts that recomputes them from the row
+// The items are numbered by one scan of all counts that recomputes them from the row
 // pointers: sums per tile of kTile rows, their scan (total in sums[blocks]), and the numbers
 // inside a tile where the items are emitted.
 __global__ void __launch_bounds__(kThreads) row_sums_k(RowSet rs, RowCount* sums) {
   const int64_t base = (int64_t)blockIdx.x * kTile + (int64_t)threadIdx.x * kItems;
-  RowCount c{0, 0, 0}, tot;
+  RowCount c{}, tot;
 #pragma unroll
   for (int j = 0; j < kItems; ++j)
-    if (base + j < rs.n_rows) c.add(rs.len(base + j), rs.L);
+    if (base + j < rs.n_rows) c.add(rs.len(base + j), rs);
   block_excl_scan(c.items, tot.items);
   block_excl_scan(c.slots, tot.slots);
   block_excl_scan(c.splits, tot.splits);
+  // at most kTile of each: the three together
+  int64_t longs;
+  block_excl_scan(c.longs[0] | c.longs[1] << 20 | c.longs[2] << 40, longs);
+#pragma unroll
+  for (int r = 0; r < 3; ++r) tot.longs[r] = longs >> (20 * r) & 0xfffff;
   if (threadIdx.x == 0) sums[blockIdx.x] = tot;
 }
 
 __global__ void __launch_bounds__(kThreads) row_sums_scan_k(RowCount* sums, int64_t m) {
-  RowCount carry{0, 0, 0};
+  RowCount carry{};
   for (int64_t b0 = 0; b0 < m; b0 += kThreads) {
     const int64_t i = b0 + threadIdx.x;
-    const RowCount v = i < m ? sums[i] : RowCount{0, 0, 0};
+    const RowCount v = i < m ? sums[i] : RowCount{};
     RowCount tot, at;
     at.items = carry.items + block_excl_scan(v.items, tot.items);
     at.slots = carry.slots + block_excl_scan(v.slots, tot.slots);
     at.splits = carry.splits + block_excl_scan(v.splits, tot.splits);
+#pragma unroll
+    for (int r = 0; r < 3; ++r) at.longs[r] = carry.longs[r] + block_excl_scan(v.longs[r], tot.longs[r]);
     if (i < m) sums[i] = at;
     carry.items += tot.items;
     carry.slots += tot.slots;
     carry.splits += tot.splits;
+#pragma unroll
+    for (int r = 0; r < 3; ++r) carry.longs[r] += tot.longs[r];
   }
   if (threadIdx.x == 0) sums[m] = carry;
 }
@@ -748,12 +762,12 @@ __global__ void __launch_bounds__(kThreads) row_emit_k(RowSet rs, const RowCount
                                                        int32_t* split_row, int32_t* split_slot_ptr) {
   const int64_t base = (int64_t)blockIdx.x * kTile + (int64_t)threadIdx.x * kItems;
   const int64_t L = rs.L;
-  RowCount c{0, 0, 0}, tot;
+  RowCount c{}, tot;
   int64_t lens[kItems];
 #pragma unroll
   for (int j = 0; j < kItems; ++j) {
     lens[j] = base + j < rs.n_rows ? rs.len(base + j) : -1;
-    c.add(lens[j], L);
+    c.add(lens[j], rs);
   }
   RowCount at = sums[blockIdx.x];
   at.items += block_excl_scan(c.items, tot.items);
@@ -764,13 +778,13 @@ __global__ void __launch_bounds__(kThreads) row_emit_k(RowSet rs, const RowCount
     const int64_t i = base + j, len = lens[j];
     if (len < 0) continue;
     RowCount next = at;
-    next.add(len, L);
+    next.add(len, rs);
     const int64_t it0 = at.items, slot0 = at.slots, sp = at.splits;
     at = next;
     BUILD_CHECK(it0 >= 0 && next.items <= total.items);
     // canonical position of the row's first entry in this set (its own entries where all are)
     const int64_t beg = cpos ? cpos[rs.rp[i]] : rs.rp[i];
-    if (len > L) {
+    if (len > rs.cut) {
       BUILD_CHECK(split_row && sp >= 0 && sp < total.splits);
       split_row[sp] = (int32_t)i;
       split_slot_ptr[sp] = (int32_t)slot0;
@@ -803,11 +817,13 @@ __global__ void item_order_k(const int64_t* order, int64_t n, const int32_t* pre
   }
 }
 
-// G lanes per item: columns and rounded values of its entries, and the value map (32-bit indices,
-// or 64-bit when wide). canon_src null: canonical positions are input entries.
+// Columns and rounded values of the items' entries, and the value map (32-bit indices, or 64-bit when
+// wide). G lanes per item, and a warp for each of the first n_first items: the segments and long rows,
+// which 8 lanes would take 64 steps for (2^18-node graph, 3.6 M entries: 44 -> 30 us). canon_src
+// null: canonical positions are input entries.
 struct ItemGatherArgs {
   const int64_t* order;
-  int64_t n;
+  int64_t n, n_first;
   const int64_t* pre_beg;
   const int64_t* item_ptr;
   const int64_t* canon_src;
@@ -827,15 +843,18 @@ struct ItemGatherArgs {
 
 template <class TB, class TIn, int G>
 __global__ void __launch_bounds__(kThreads) item_gather_k(ItemGatherArgs a) {
-  const int sub = threadIdx.x & (G - 1);
   const TIn* vals = reinterpret_cast<const TIn*>(a.vals);
   unsigned long long n_sub = 0;
-  for (int64_t q = ((int64_t)blockIdx.x * kThreads + threadIdx.x) / G; q < a.n;
-       q += (int64_t)gridDim.x * (kThreads / G)) {
+  constexpr int W = 32 / G;  // groups per warp
+  for (int64_t g = ((int64_t)blockIdx.x * kThreads + threadIdx.x) / G; g < a.n + (W - 1) * a.n_first;
+       g += (int64_t)gridDim.x * (kThreads / G)) {
+    const bool first = W > 1 && g < W * a.n_first;
+    const int64_t q = first ? g / W : g - (W - 1) * a.n_first;
+    const int sub = threadIdx.x & (first ? 31 : G - 1), step = first ? 32 : G;
     const int64_t b = a.pre_beg[a.order[q]];
     const int64_t d0 = a.item_ptr[q], len = a.item_ptr[q + 1] - d0;
     BUILD_CHECK(b >= 0 && b + len <= a.n_canon && d0 >= 0 && d0 + len <= a.total);
-    for (int64_t e = sub; e < len; e += G) {
+    for (int64_t e = sub; e < len; e += step) {
       const int64_t k = a.canon_src ? a.canon_src[b + e] : b + e;
       a.col[d0 + e] = a.ci[k];
       const TB x = stored_value<TB>(vals[k], a.scale, a.scale_f);
@@ -938,7 +957,7 @@ cudaError_t launch_tile_values(const TileArgs& a, cudaStream_t s) {
 template <class TB, class TIn>
 cudaError_t launch_item_gather(const ItemGatherArgs& a, cudaStream_t s) {
   const bool narrow = a.total < 24 * a.n;
-  const int64_t lanes = a.n * (narrow ? 8 : 32);
+  const int64_t lanes = narrow ? a.n * 8 + a.n_first * 24 : a.n * 32;
   const unsigned blocks = (unsigned)std::max<int64_t>(1, std::min<int64_t>((lanes + kThreads - 1) / kThreads, 152 * 16));
   if (narrow) item_gather_k<TB, TIn, 8><<<blocks, kThreads, 0, s>>>(a);
   else item_gather_k<TB, TIn, 32><<<blocks, kThreads, 0, s>>>(a);
@@ -1004,19 +1023,24 @@ loops_status build_csr_set(loops_plan_s* p, const DevCsrIn& A, const int64_t* re
   int64_t& bytes = p->dev.device_bytes;
   const int64_t n = A.n_rows;
   if (n == 0) return LOOPS_OK;
-  const RowSet rs{A.rp, is_bcsr, rowlen1, n, std::max<int64_t>(p->split_len, 1), p->br, which};
+  const int team_base = p->team_len > 0 ? bit_width((uint64_t)p->team_len) - 1 : -1;  // the class of team_len - 1
+  const RowSet rs{A.rp, is_bcsr, rowlen1, n, std::max<int64_t>(p->split_len, 1), std::max<int64_t>(p->cut_len, 1), p->br,
+                  which, team_base};
   const int64_t row_blocks = (n + kTile - 1) / kTile;
   RowCount* sums = ar.get<RowCount>(row_blocks + 1);
   NEED(sums);
   row_sums_k<<<(unsigned)row_blocks, kThreads, 0, s>>>(rs, sums);
   row_sums_scan_k<<<1, kThreads, 0, s>>>(sums, row_blocks);
   TRY(cudaGetLastError());
-  RowCount total{0, 0, 0};
+  RowCount total{};
   TRY(to_host(&total, sums + row_blocks, s));
   const int64_t n_it = total.items;
   cd.n_items = n_it;
   cd.n_slots = total.slots;
   cd.n_split = total.splits;
+  for (int r = 0; r < 3; ++r) cd.n_long[r] = total.longs[r];
+  cd.team_len = p->team_len;
+  limit_teams(cd, N, p->dtype);
   if (n_it == 0) return LOOPS_OK;
   uint64_t* ikey = ar.get<uint64_t>(n_it);
   uint64_t* ikey2 = ar.get<uint64_t>(n_it);
@@ -1046,9 +1070,11 @@ loops_status build_csr_set(loops_plan_s* p, const DevCsrIn& A, const int64_t* re
   item_order_k<<<grid_for(n_it), kThreads, 0, s>>>(ival, n_it, pre_row, pre_len, cd.item_row, dlen);
   TRY(cudaGetLastError());
   TRY(excl_scan<int64_t>(dlen, cd.item_ptr, n_it, true, ar, s));
+  const int64_t n_first =
+      LOOPS_CSR_ITEMS_BY_LENGTH ? total.slots + total.longs[0] + total.longs[1] + total.longs[2] : 0;
   cd.nnz = n_canon;  // the set's rows hold exactly its entries
   if (n_canon) {
-    const ItemGatherArgs ga{ival, n_it, pre_beg, cd.item_ptr, csrc, n_canon, n_canon, A.ci, A.vals, p->scale,
+    const ItemGatherArgs ga{ival, n_it, n_first, pre_beg, cd.item_ptr, csrc, n_canon, n_canon, A.ci, A.vals, p->scale,
                             scale_f32(p->scale), (float)tiny, remap, cd.col, cd.val, csr_src ? *csr_src : nullptr,
                             wide ? 1 : 0, n_sub};
     TRY(dispatch_item_gather(p->dtype, A.vals_f32, ga, s));
