@@ -221,17 +221,19 @@ void destroy_plan(loops_plan_s* p) {
 // the segments of rows above kDefaultCutLen entries, and what the teams of shorter rows are sized by.
 // A group works through its entries a few at a time, so the longest chain bounds a small problem's
 // time (512 entries: 50 to 80 us). Only rows above kDefaultCutLen become segments: their partial
-// sums are the plan's memory, which calls on two streams would share. The length follows the entries per resident lane group (about
-// 2^18 lanes on the GPU; a group has the lanes of two 16-byte vectors each, 8 to 32), in [64, 512].
+// sums are the plan's memory, which calls on two streams would share. The length follows the entries
+// per resident lane group (about 2^18 lanes on the GPU; a group has the lanes of two 16-byte vectors
+// each, 8 to 32), in [64, 512], and is raised until nnz / length rows of partial sums fit kMaxPartialBytes.
 // Measured against one group for every row of up to 512 entries: graphs of 4,000 and 30,000 nodes (N =
 // 64, 128, FP32) 80 -> 19 and 96 -> 23 us; with segments of 64 for every size the GCN layer (N = 256, FP32)
-// loses 7 %.
+// loses 7 %. Counting the lanes of all column chunks of a wide N (50,000 nodes, N = 384, FP32: 256 for 128
+// entries) gives 124 us instead of 103.
+constexpr int64_t kMaxPartialBytes = (int64_t)64 << 20;
 static int32_t default_split_len(int64_t nnz, int64_t N, loops_dtype dtype) {
-  const int64_t row_bytes = N * dense_elem_bytes(dtype);
-  int64_t lanes = 8;
-  while (lanes < 32 && lanes * 32 < row_bytes) lanes *= 2;
+  const int64_t lanes = std::min<int64_t>(row_lanes(N, dtype), 32);
+  const double partials = (double)nnz * (double)N * (dtype == LOOPS_F64 ? 8 : 4);
   int32_t len = 64;
-  while (len < 512 && len < nnz * lanes >> 18) len *= 2;
+  while (len < 512 && (len < nnz * lanes >> 18 || partials / len > (double)kMaxPartialBytes)) len *= 2;
   return len;
 }
 

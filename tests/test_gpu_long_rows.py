@@ -91,3 +91,18 @@ def test_calls_of_one_plan_on_two_streams(loops_lib, fmt, N):
     for i in range(2):
         for C, (dB, dv) in got[i]:
             assert torch.equal(C, ref[i][0]) and torch.equal(dB, ref[i][1][0]) and torch.equal(dv, ref[i][1][1])
+
+
+@pytest.mark.parametrize("on_device", [False, True])
+@pytest.mark.parametrize("fmt,N,segment", [("f32", 64, 64), ("f32", 512, 128), ("bf16", 2048, 128), ("f64", 1024, 128),
+                                           ("f32", 4096, 256), ("f32", 1 << 16, 512)])
+def test_default_segments_of_wide_rows(loops_lib, fmt, N, segment, on_device):
+    # one row of 10^6 entries: the segments' partial sums (n_segments x N) stay small for any N
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    nnz = 1_000_000
+    A = rows_of(np.array([5, nnz, 0]), 700, 1)
+    info = loops_lib.Plan(A, N, fmt, tau=math.inf, build_on_device=on_device).info()
+    assert info["n_segments"] == -(-nnz // segment)
+    plan = loops_lib.Plan(A, N, fmt, tau=math.inf, split_len=512, build_on_device=on_device)
+    assert info["device_bytes"] <= plan.info()["device_bytes"] + (65 << 20)
