@@ -670,7 +670,7 @@ static loops_status plan_batched(const loops_csr* As, const int64_t* Ns, int32_t
   o.tile_min = 0;
   o.want_backward = 0;
   o.contiguous_split = 0;
-  if (o.split_len <= 0) o.split_len = kDefaultCutLen;  // one launch for all matrices: no need to cut small ones finer
+  if (o.split_len <= 0) o.split_len = 512;  // one launch for all matrices: no need to cut small ones finer
   int32_t br;
   loops_status st = resolve_block_rows(dtype, o, &br);
   if (st) return st;
