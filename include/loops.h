@@ -106,7 +106,9 @@ typedef struct {
   int32_t split_len;      /* CSR rows longer than this are split in segments of this length; 0 =
                              default: rows above 512 entries, in segments of 64 to 512 by size */
   int32_t tile_min;
-  int32_t reserved[5];
+  int32_t test_wide_maps; /* test hook: 64-bit value maps (loops_plan_set_values), which otherwise only
+                             matrices of 2^31 entries or BCSR slots and more take; 0: by size */
+  int32_t reserved[4];
 } loops_plan_opts;
 
 typedef struct loops_plan_s* loops_plan_t;

@@ -55,7 +55,7 @@ class _Opts(ctypes.Structure):
     _fields_ = [("tau", ctypes.c_double), ("block_rows", ctypes.c_int32),
                 ("contiguous_split", ctypes.c_int32), ("r_boundary", ctypes.c_int64),
                 ("want_backward", ctypes.c_int32), ("split_len", ctypes.c_int32),
-                ("tile_min", ctypes.c_int32), ("reserved", ctypes.c_int32 * 5)]
+                ("tile_min", ctypes.c_int32), ("test_wide_maps", ctypes.c_int32), ("reserved", ctypes.c_int32 * 4)]
 
 
 class _Info(ctypes.Structure):

@@ -326,7 +326,7 @@ loops_status upload_value_maps(loops_plan_s* p, const std::vector<int64_t>* rema
   }
   m.n_csr = (int64_t)csr_src.size();
   m.n_slots = n_slots;
-  m.wide = value_maps_wide(nnz, n_slots);
+  m.wide = p->opts.test_wide_maps || value_maps_wide(nnz, n_slots);
   auto up = [&](void** dst, const std::vector<int64_t>& v) -> loops_status {
     if (m.wide) return dev_upload((int64_t**)dst, v.data(), v.size(), m.bytes);
     const std::vector<int32_t> w(v.begin(), v.end());

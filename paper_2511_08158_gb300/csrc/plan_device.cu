@@ -1179,7 +1179,7 @@ loops_status build_part_device(loops_plan_s* p, const DevCsrIn& A, const int64_t
     if (want_maps) {
       free_value_maps(m);
       m.n_csr = nnz;
-      m.wide = value_maps_wide(nnz, 0);
+      m.wide = p->opts.test_wide_maps || value_maps_wide(nnz, 0);
     }
     const loops_status st = build_csr_set(p, A, remap, 0, nullptr, nullptr, nullptr, nullptr, nnz, N, tiny, n_sub,
                                           want_maps ? &m.csr_src : nullptr, m.wide, ar, s);
@@ -1395,7 +1395,7 @@ loops_status build_part_device(loops_plan_s* p, const DevCsrIn& A, const int64_t
     free_value_maps(m);
     m.n_csr = nnz0;
     m.n_slots = n_fslots;
-    m.wide = value_maps_wide(nnz, n_fslots);
+    m.wide = p->opts.test_wide_maps || value_maps_wide(nnz, n_fslots);
   }
   loops_status st;
   if ((st = build_csr_set(p, A, remap, 0, is_bcsr, rowlen1, c0, src0, nnz0, N, tiny, n_sub,
