@@ -686,10 +686,12 @@ __global__ void __launch_bounds__((CsrBlock<G, TEAM>::kThreads), (BwdShape<Tr, V
     }
   }
   if constexpr (Tr::kScaled) {
-    if (__any_sync(gmask, lossy))  // also orders the stores above before those that replace them
+    if (__any_sync(gmask, lossy)) {
+      __syncwarp(gmask);  // the stores of the loop above come before those that replace them
       weighted_dots<Tr, G, TEAM>(a.col + beg, w.src + beg, len, sh, sub, gmask, reinterpret_cast<const TB*>(a.B), a.ldb,
                                  reinterpret_cast<const TB*>(w.B) + (int64_t)j * w.ldb, w.dc_scale, w.b_scale, a.N,
                                  dvals);
+    }
   }
   if constexpr (TEAM) {
     if (sh.log_size >= 0 && !team_sum<G>(sh, acc)) return;
