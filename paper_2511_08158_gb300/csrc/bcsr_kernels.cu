@@ -15,6 +15,9 @@
 //             pipe, slower, and multiplies the tiles' zeros).
 //   F32       CUDA-core register-blocked outer product (TF32 MMA would not meet FP32
 //             accuracy): a group of lanes owns B_r x 4*G outputs and updates them per tile.
+#include <algorithm>
+#include <type_traits>
+
 #include "device_common.cuh"
 #include "loops_internal.h"
 
@@ -74,20 +77,57 @@ __device__ __forceinline__ void ldsm_x2_trans(uint32_t addr, uint32_t& r0, uint3
                : "=r"(r0), "=r"(r1) : "r"(addr));
 }
 
-// One warp per work unit and CT = 8 * NF columns, kHmmaUnits independent warps per CTA. BULK: B rows
-// are fetched with cp.async.bulk (needs 16-byte aligned rows and a multiple-of-8 N); otherwise the
-// lanes copy them element-wise.
+// One warp per work unit and CT = 8 * NF columns, kHmmaUnits independent warps per CTA. COPY: B rows
+// are fetched with cp.async.bulk (needs 16-byte aligned rows and a multiple-of-8 N), or the lanes copy
+// them, in aligned pairs (even N and rows on 4 bytes) or single elements.
 //
 // Bound by the latency of a unit's chain (unit, columns, B rows, C): most units have a few groups, so
 // what counts is units in flight per SM. A warp of its own needs no CTA barrier and kStages = 2
 // stages let more of them in, all of a short unit's rows in flight at once. Block mix, N = 64,
 // BF16 (32,780 units of two groups), whole SpMM: 237 -> 197 us, against four warps on 16 columns each
 // with a barrier per group and four stages; three stages 218 us, N = 256 on 2^18 rows 178 -> 164 us.
+//
+// Lanes that copy must not wait for one load after another: a stage's loads go out together, the first
+// two stages' before any store, later ones before the MMAs of the group they replace. At most 32
+// columns per warp, so that they fit the registers. 65,536 rows of two dense 16 x 16 blocks, FP16,
+// against four warps per unit with a barrier per group: N = 100 23.1 -> 19.2 us, 250 43.5 -> 35.5,
+// 61 16.8 -> 16.8, 99 25.0 -> 27.1 (one element at a time 43.6); with half the rows scattered (a CSR part beside)
+// 1.6 to 2.8 times as fast, units of 12 groups 2 to 2.5. Tiles of 64 columns: N = 36, 12 groups 48.8 ->
+// 24.3 us against 19.1; of 16: N = 250 41.7 us.
 constexpr int kStages = 2;
 constexpr int kHmmaUnits = 2;
 
-template <class T, int NF, bool BULK>
+enum class RowCopy { kElements, kPairs, kBulk };
+
+// A lane's share of the 16 rows of a stage where they are not bulk copies: Words (an element, or an
+// aligned pair of them) lane, lane + 32, ... of the stage, zeros for padding tiles (column -1, held by lane k
+// for row k) and past `width`. All of a lane's loads are in flight together, and apart from their stores.
+template <class T, int CT, class Word>
+struct RowShare {
+  static constexpr int W = sizeof(Word) / sizeof(T), kWords = CT / W, kLoads = 16 * kWords / 32;
+  Word x[kLoads];
+  __device__ __forceinline__ void load(const T* Bp, int64_t ldb, int32_t c_lane, int width, int lane) {
+#pragma unroll
+    for (int d = 0; d < kLoads; ++d) {
+      const int i = d * 32 + lane, n = i % kWords * W;
+      const int32_t c = __shfl_sync(0xffffffffu, c_lane, i / kWords);
+      x[d] = 0;
+      if (c >= 0 && n < width) x[d] = __ldg(reinterpret_cast<const Word*>(Bp + (int64_t)c * ldb + n));
+    }
+  }
+  template <int RS>
+  __device__ __forceinline__ void store(T (*st)[RS], int lane) const {
+#pragma unroll
+    for (int d = 0; d < kLoads; ++d) {
+      const int i = d * 32 + lane;
+      *reinterpret_cast<Word*>(&st[i / kWords][i % kWords * W]) = x[d];
+    }
+  }
+};
+
+template <class T, int NF, RowCopy COPY>
 __global__ void __launch_bounds__(kHmmaUnits * 32) bcsr_hmma(BcsrKArgs a) {
+  constexpr bool BULK = COPY == RowCopy::kBulk;
   constexpr int CT = 8 * NF;
   constexpr int RS = CT + 8;  // smem row stride in elements (+16 B: conflict-free ldmatrix)
   __shared__ __align__(128) T sB_all[kHmmaUnits][kStages][16][RS];
@@ -122,7 +162,7 @@ __global__ void __launch_bounds__(kHmmaUnits * 32) bcsr_hmma(BcsrKArgs a) {
   // once. The caller has synchronised the warp since the stage was last read.
   auto issue = [&](int g) {
     const int s = g % kStages;
-    if (BULK) {
+    if constexpr (BULK) {
       const uint32_t row_bytes = (uint32_t)width * sizeof(T);
       const int32_t c = lane < 16 ? cols[g * 16 + lane] : -1;
       if (lane < 16 && c < 0) {
@@ -137,12 +177,6 @@ __global__ void __launch_bounds__(kHmmaUnits * 32) bcsr_hmma(BcsrKArgs a) {
         fence_proxy_async_smem();
         bulk_g2s(&sB[s][lane][0], Bp + (int64_t)c * a.ldb + n0, row_bytes, &bar[s]);
       }
-    } else {
-      for (int i = lane; i < 16 * CT; i += 32) {
-        const int k = i / CT, n = i % CT;
-        const int32_t c = cols[g * 16 + k];
-        sB[s][k][n] = (c >= 0 && n < width) ? Bp[(int64_t)c * a.ldb + n0 + n] : T(0.f);
-      }
     }
   };
 
@@ -152,10 +186,24 @@ __global__ void __launch_bounds__(kHmmaUnits * 32) bcsr_hmma(BcsrKArgs a) {
 #pragma unroll
     for (int i = 0; i < 4; ++i) acc[f][i] = 0.f;
 
-  for (int g = 0; g < min(n_groups, kStages); ++g) issue(g);
+  using Word = std::conditional_t<COPY == RowCopy::kPairs, uint32_t, uint16_t>;
+  RowShare<T, CT, Word> rows;
+  auto load_rows = [&](int g, RowShare<T, CT, Word>& x) {
+    x.load(Bp + n0, a.ldb, lane < 16 && g < n_groups ? cols[g * 16 + lane] : -1, width, lane);
+  };
+  if constexpr (BULK) {
+    for (int g = 0; g < min(n_groups, kStages); ++g) issue(g);
+  } else {
+    RowShare<T, CT, Word> first;
+    load_rows(0, first);
+    load_rows(1, rows);
+    first.store(sB[0], lane);
+    rows.store(sB[1], lane);
+  }
   for (int g = 0; g < n_groups; ++g) {
     const uint4 af = __ldg(Af + (int64_t)g * 32 + lane);
     const int s = g % kStages;
+    if constexpr (!BULK) load_rows(g + kStages, rows);
     if (BULK) {
       const bool ok = mbar_wait_bounded(&bar[s], (uint32_t)((g / kStages) & 1), a.max_polls);
       if (__any_sync(0xffffffffu, !ok)) {
@@ -192,7 +240,11 @@ __global__ void __launch_bounds__(kHmmaUnits * 32) bcsr_hmma(BcsrKArgs a) {
       }
     }
     __syncwarp();  // every lane has read the stage
-    if (g + kStages < n_groups) issue(g + kStages);
+    if constexpr (BULK) {
+      if (g + kStages < n_groups) issue(g + kStages);
+    } else {
+      rows.store(sB[s], lane);
+    }
   }
   // epilogue: acc[f] = C rows (q, q + 8) x columns (2t, 2t + 1) of fragment f
   const int q = lane >> 2, t = lane & 3;
@@ -236,26 +288,37 @@ __global__ void __launch_bounds__(kHmmaUnits * 32) bcsr_hmma(BcsrKArgs a) {
   }
 }
 
-template <class T, int NF>
-cudaError_t launch_hmma_cfg(const BcsrKArgs& a, bool bulk, cudaStream_t s) {
+template <class T, int NF, RowCopy COPY>
+cudaError_t launch_hmma_cfg(const BcsrKArgs& a, cudaStream_t s) {
   constexpr int CT = 8 * NF;
-  dim3 grid((unsigned)((a.n_units + kHmmaUnits - 1) / kHmmaUnits), (unsigned)((a.N + CT - 1) / CT));
-  if (bulk) bcsr_hmma<T, NF, true><<<grid, kHmmaUnits * 32, 0, s>>>(a);
-  else bcsr_hmma<T, NF, false><<<grid, kHmmaUnits * 32, 0, s>>>(a);
+  const dim3 grid((unsigned)((a.n_units + kHmmaUnits - 1) / kHmmaUnits), (unsigned)((a.N + CT - 1) / CT));
+  bcsr_hmma<T, NF, COPY><<<grid, kHmmaUnits * 32, 0, s>>>(a);
   return cudaGetLastError();
 }
 
 // Column tile of a warp: the plan's bcsr_ntile when the autotuner set it (32, 64 or 128), else
-// the smallest of 8 .. 128 that covers N.
+// the smallest of 8 .. 128 that covers N; at most WIDEST (the reasons stand at the kernel).
+template <class T, RowCopy COPY, int WIDEST>
+cudaError_t launch_hmma_copy(const BcsrKArgs& a, int ntile, cudaStream_t s) {
+  const int64_t ct = std::min<int64_t>(ntile > 0 ? ntile : a.N, WIDEST);
+  if (ct <= 8) return launch_hmma_cfg<T, 1, COPY>(a, s);
+  if (ct <= 16) return launch_hmma_cfg<T, 2, COPY>(a, s);
+  if constexpr (WIDEST > 16) {
+    if (ct <= 32) return launch_hmma_cfg<T, 4, COPY>(a, s);
+  }
+  if constexpr (WIDEST > 32) return ct <= 64 ? launch_hmma_cfg<T, 8, COPY>(a, s) : launch_hmma_cfg<T, 16, COPY>(a, s);
+  return cudaErrorInvalidValue;
+}
+
 template <class T>
 cudaError_t launch_hmma(const BcsrKArgs& a, int ntile, cudaStream_t s) {
-  const bool bulk = (a.N % 8 == 0) && ((uintptr_t)a.B % 16 == 0) && ((a.ldb * 2) % 16 == 0);
-  const int64_t ct = ntile > 0 ? ntile : (a.N <= 8 ? 8 : a.N <= 16 ? 16 : a.N <= 32 ? 32 : a.N <= 64 ? 64 : 128);
-  if (ct <= 8) return launch_hmma_cfg<T, 1>(a, bulk, s);
-  if (ct <= 16) return launch_hmma_cfg<T, 2>(a, bulk, s);
-  if (ct <= 32) return launch_hmma_cfg<T, 4>(a, bulk, s);
-  if (ct <= 64) return launch_hmma_cfg<T, 8>(a, bulk, s);
-  return launch_hmma_cfg<T, 16>(a, bulk, s);
+  if (a.N % 8 == 0 && (uintptr_t)a.B % 16 == 0 && (a.ldb * 2) % 16 == 0)
+    return launch_hmma_copy<T, RowCopy::kBulk, 128>(a, ntile, s);
+  if (a.N % 2 == 0 && (uintptr_t)a.B % 4 == 0 && a.ldb % 2 == 0)
+    return launch_hmma_copy<T, RowCopy::kPairs, 32>(a, ntile, s);
+  // single elements: the tile that leaves fewer columns idle (N = 33: 16.1 us with 32, 14.5 with 16; 61: 16.8 and 17.2)
+  if ((a.N - 1) % 32 < 16) return launch_hmma_copy<T, RowCopy::kElements, 16>(a, ntile, s);
+  return launch_hmma_copy<T, RowCopy::kElements, 32>(a, ntile, s);
 }
 
 // ------------------------------------------------------------------ F64: FP64 FMAs on the entries
@@ -333,7 +396,7 @@ __global__ void __launch_bounds__(128) bcsr_f64(BcsrKArgs a) {
           load2(brow, n + 2, x[p][2], x[p][3]);
         }
       }
-      // a row without a next entry adds zeros: w * 0 with its own w, which is finite
+      // a row without a next entry adds zeros: 0 * 0
 #pragma unroll
       for (int p = 0; p < NP; ++p)
 #pragma unroll
