@@ -97,15 +97,21 @@ struct Slice {
   }
 };
 
-constexpr int kNoAllocWarps = 8;
+// warps per block; four of FP64 spread a small call's FP64 work over more SMs
+template <class Tr>
+constexpr int kNoAllocWarps = std::is_same<Tr, TrF64>::value ? 4 : 8;
 constexpr int kNoAllocU = 4;  // entries in flight per group
 
 // Bound by the gathers of B rows. The chunk's columns and values are staged in shared memory
 // first, so that the gathers depend on no global load, and kNoAllocU of them are in flight per
 // group. 65,536 rows of 32 entries, N = 64, FP32: 65 us a call (both kernels), against 196 us with
 // one gather in flight, the entries read per 32 columns, and four binary searches per chunk.
+// FP64 is bound by the FP64 pipe, where an instruction costs the same for one live lane as for 32: no
+// FMA past a row's end, sums over only the groups that had an entry, and up to N = 32 one column per lane,
+// since vectors of two mean twice the instructions and more groups to sum. 200,000 rows of 4 entries, N =
+// 16, 93 -> 61 us (vectors 158); 30,000 of 33, N = 8, 102 -> 35 us (vectors 55).
 template <class Tr, int G, int CP, bool VEC>
-__global__ void __launch_bounds__(kNoAllocWarps * 32) noalloc_chunks(NoAllocArgs a) {
+__global__ void __launch_bounds__(kNoAllocWarps<Tr> * 32) noalloc_chunks(NoAllocArgs a) {
   using TB = typename Tr::TB;
   using TAcc = typename Tr::TAcc;
   using TC = typename Tr::TC;
@@ -114,10 +120,11 @@ __global__ void __launch_bounds__(kNoAllocWarps * 32) noalloc_chunks(NoAllocArgs
   constexpr int NC = S::kCols;
   constexpr int NG = 32 / G;
   constexpr int U = kNoAllocU;
-  __shared__ int32_t s_col[kNoAllocWarps][kChunk];
-  __shared__ TV s_val[kNoAllocWarps][kChunk];
+  constexpr bool F64 = std::is_same<Tr, TrF64>::value;
+  __shared__ int32_t s_col[kNoAllocWarps<Tr>][kChunk];
+  __shared__ TV s_val[kNoAllocWarps<Tr>][kChunk];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t c = (int64_t)blockIdx.x * kNoAllocWarps + warp;
+  const int64_t c = (int64_t)blockIdx.x * kNoAllocWarps<Tr> + warp;
   if (c >= a.n_chunks) return;
   const int sub = lane & (G - 1), grp = lane / G;
   const int64_t e0 = c * kChunk;
@@ -147,7 +154,7 @@ __global__ void __launch_bounds__(kNoAllocWarps * 32) noalloc_chunks(NoAllocArgs
   TAcc* head = reinterpret_cast<TAcc*>(a.scratch);
   TAcc* tail = head + a.n_chunks * a.N;
 
-  // sum over the chunk's entries [k0, k1), in every lane of the group's columns
+  // sum over the chunk's entries [k0, k1), in the lanes of group 0
   auto dot = [&](int k0, int k1, TAcc (&acc)[NC]) {
 #pragma unroll
     for (int i = 0; i < NC; ++i) acc[i] = TAcc(0);
@@ -162,8 +169,14 @@ __global__ void __launch_bounds__(kNoAllocWarps * 32) noalloc_chunks(NoAllocArgs
           av[u] = cj >= 0 ? val[k] : TV(0);
           bv[u] = ldg16_if(ok[0] && cj >= 0, bl + (int64_t)cj * a.ldb);
         }
+        if (!F64 || kb + NG * U <= k1) {
 #pragma unroll
-        for (int u = 0; u < U; ++u) fma_vec<Tr>(acc, bv[u], av[u]);
+          for (int u = 0; u < U; ++u) fma_vec<Tr>(acc, bv[u], av[u]);
+        } else {
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            if (u == 0 || kb + u * NG < k1) fma_vec<Tr>(acc, bv[u], av[u]);
+        }
       } else {
         TB bv[U][NC];
         bool live[U];
@@ -180,6 +193,7 @@ __global__ void __launch_bounds__(kNoAllocWarps * 32) noalloc_chunks(NoAllocArgs
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
+          if (F64 && u > 0 && kb + u * NG >= k1) break;
           const TAcc w = value_of<Tr>(av[u]);
 #pragma unroll
           for (int i = 0; i < NC; ++i)
@@ -188,9 +202,11 @@ __global__ void __launch_bounds__(kNoAllocWarps * 32) noalloc_chunks(NoAllocArgs
       }
     }
 #pragma unroll
-    for (int off = G; off < 32; off <<= 1)
+    for (int off = G; off < 32; off <<= 1) {
+      if (F64 && off >= (k1 - k0) * G) break;  // the groups from off / G on had no entry
 #pragma unroll
       for (int i = 0; i < NC; ++i) acc[i] += __shfl_xor_sync(0xffffffffu, acc[i], off);
+    }
   };
 
   // rows owned by this chunk: first entry in [e0, e1) (the last chunk also owns trailing
@@ -285,12 +301,13 @@ __global__ void __launch_bounds__(256) noalloc_fixup(NoAllocArgs a) {
 
 template <class Tr>
 cudaError_t launch_noalloc_t(const NoAllocArgs& a, cudaStream_t s) {
-  const unsigned gx = (unsigned)((a.n_chunks + kNoAllocWarps - 1) / kNoAllocWarps);
+  constexpr int kWarps = kNoAllocWarps<Tr>;
+  const unsigned gx = (unsigned)((a.n_chunks + kWarps - 1) / kWarps);
   auto go = [&](auto g_tag, auto cp_tag, auto vec_tag) {
     constexpr int G = decltype(g_tag)::value, CP = decltype(cp_tag)::value;
     constexpr bool VEC = decltype(vec_tag)::value;
     constexpr int width = Slice<Tr, G, CP, VEC>::kWidth;
-    noalloc_chunks<Tr, G, CP, VEC><<<dim3(gx, (unsigned)((a.N + width - 1) / width)), kNoAllocWarps * 32, 0, s>>>(a);
+    noalloc_chunks<Tr, G, CP, VEC><<<dim3(gx, (unsigned)((a.N + width - 1) / width)), kWarps * 32, 0, s>>>(a);
   };
   using std::integral_constant;
   using C1 = integral_constant<int, 1>;
@@ -300,7 +317,8 @@ cudaError_t launch_noalloc_t(const NoAllocArgs& a, cudaStream_t s) {
   const int64_t eb = sizeof(typename Tr::TB), ec = sizeof(typename Tr::TC);
   const bool vec = a.N % Tr::kVE == 0 && (uintptr_t)a.B % 16 == 0 && (uintptr_t)a.C % 16 == 0 &&
                    (a.ldb * eb) % 16 == 0 && (a.ldc * ec) % 16 == 0;
-  if (vec) {
+  const bool single = std::is_same<Tr, TrF64>::value && a.N <= 32;  // the reasons stand at the kernel
+  if (vec && !single) {
     const int64_t nvec = a.N / Tr::kVE;
     if (nvec <= 1) go(C1(), C1(), std::true_type());
     else if (nvec <= 2) go(integral_constant<int, 2>(), C1(), std::true_type());
@@ -314,7 +332,7 @@ cudaError_t launch_noalloc_t(const NoAllocArgs& a, cudaStream_t s) {
     go(integral_constant<int, 16>(), C1(), std::false_type());
   } else if (a.N <= 32) {
     go(C32(), C1(), std::false_type());
-  } else if (a.N <= 64) {
+  } else if (a.N <= 64 || a.n_chunks <= 2048) {  // few chunks: more slices, so that more warps run
     go(C32(), integral_constant<int, 2>(), std::false_type());
   } else {
     go(C32(), integral_constant<int, 4>(), std::false_type());
