@@ -169,7 +169,7 @@ __device__ __forceinline__ void csr_item(const BatchDesc& d, int64_t item, int s
 #pragma unroll
           for (int p = 0; p < VPL; ++p) {
             if constexpr (FULL) bv[u][p] = ldg16(bl[p] + cj * ldb);
-            else bv[u][p] = ldg16_if(colok[p], bl[p] + cj * ldb);
+            else bv[u][p] = colok[p] ? ldg16(bl[p] + cj * ldb) : make_uint4(0, 0, 0, 0);  // (as ldg16_if: N = 24 9 % slower)
           }
         }
 #pragma unroll
@@ -254,30 +254,41 @@ __global__ void __launch_bounds__(256, csr_min_blocks<Tr>()) batched_csr(const B
 }
 
 // ------------------------------------------------------------------ F32 BCSR units
-// Tiles in flight and resident blocks per SM (register caps). The units wait on their loads: with
-// B_r 8 two tiles at 4 blocks beat four at 3 (batch of 128 matrices 755 -> 724 us, with the
-// unpredicated loads; N = 16, 32, 64 of the 512-matrix batch 119, 234, 352 -> 112, 222, 323 us) and
-// three at either; one tile, or two at 5 blocks, spill (1.4x the call). B_r 16 holds 64
-// accumulators per lane at 2 blocks: three tiles (batch of 128 matrices 762 us; two 809, one 825).
-template <int BR>
+// Tiles in flight, resident blocks per SM (register caps) and the form of a full batch's loads: plain
+// with 32-bit row offsets, or under a predicate with 64-bit ones. The units wait on their loads and the
+// caps are tight, so the compiler's spills decide; every instance was timed alone, 24 and 64 matrices
+// (banded, and two dense blocks per 16 rows), against four tiles (B_r 16: two) at 3 (2) blocks under predicates:
+// * B_r 8, lanes that cover N: two tiles at 4 blocks, plain (84 to 100 bytes spilled): N = 16, 32, 64
+//   1.02 to 1.2 times as fast (banded, 64 matrices, N = 64 725 -> 647 us); three tiles 0.97 to 1.07,
+//   four at 3 blocks 0.85 to 1.0.
+// * B_r 8, N covered partly: predicates, B's address from the descriptor each time (108 spilled; 120 with
+//   the address kept: 0.93 to 0.99): N = 24, 36 1.01 to 1.06; plain 0.94 to 1.0.
+// * B_r 8, 32 lanes: predicates, nothing spilled: N = 100, 128 1.01 to 1.05; plain 0.90 to 0.99.
+// * B_r 16: predicates, two tiles, nothing spilled (plain, three tiles: N = 24 to 64 0.91 to 1.02; predicates,
+//   three tiles 0.86 to 0.95); 32 lanes three tiles: N = 100, 128 1.05 to 1.09 (plain 1.03 to 1.08).
+template <int BR, int G, bool FULL>
 struct FfmaShape {
-  static constexpr int kTiles = BR == 16 ? 3 : 2;
-  static constexpr int kMinBlocks = BR == 16 ? 2 : 4;
+  static constexpr bool kPlain = BR == 8 && FULL && G < 32;
+  static constexpr bool kReloadB = BR == 8 && !FULL && G < 32;
+  static constexpr int kTiles = BR == 16 && G == 32 ? 3 : 2;
+  static constexpr int kMinBlocks = BR == 8 ? 4 : 2;
 };
 
 // One F32 BCSR unit (B_r rows, tile-major values) for a group of G lanes, 4 columns per lane;
 // T tiles' B vectors and A values are loaded before their FMAs.
 template <int BR, int G, bool FULL>
 __device__ __forceinline__ void ffma_unit(const BatchDesc& d, int64_t u, int sub) {
-  constexpr int T = FfmaShape<BR>::kTiles;
+  constexpr int T = FfmaShape<BR, G, FULL>::kTiles;
+  constexpr bool PLAIN = FfmaShape<BR, G, FULL>::kPlain;
   const int32_t b = d.unit_block[u];
   const int64_t rb = d.rb_id[b];
   const int64_t t0 = d.unit_t0[u], t1 = d.unit_t1[u];
   const int32_t slot = d.unit_slot[u];
   const float* __restrict__ Av = reinterpret_cast<const float*>(d.tile_val);
+  const float* __restrict__ Bp = reinterpret_cast<const float*>(d.B);
   const int64_t n = (int64_t)sub * 4;
-  const bool colok = FULL || n < d.N;
-  const float* __restrict__ bl = reinterpret_cast<const float*>(d.B) + n;
+  const bool colok = PLAIN || n < d.N;
+  const float* __restrict__ bl = Bp + n;
   const uint32_t ldb = (uint32_t)d.ldb;  // the batched call keeps every B below 2^31 elements
   float acc[BR][4];
 #pragma unroll
@@ -302,17 +313,23 @@ __device__ __forceinline__ void ffma_unit(const BatchDesc& d, int64_t u, int sub
 #pragma unroll
     for (int q = 0; q < T; ++q) cc[q] = base + q < t1 ? __ldg(d.tile_col + base + q) : -1;
   };
-  // F32 blocks have no padding tiles, so every tile of a full batch has a column
-  auto load_tile = [&](int64_t tt, int32_t c, uint4& v, uint4 (&w)[BR / 4]) {
-    if constexpr (FULL) v = ldg16(bl + (uint32_t)c * ldb);
-    else v = ldg16_if(colok, bl + (uint32_t)c * ldb);
-#pragma unroll
-    for (int r4 = 0; r4 < BR / 4; ++r4) w[r4] = ldg16(Av + tt * BR + r4 * 4);
-  };
-  auto load_tile_if = [&](bool live, int64_t tt, int32_t c, uint4& v, uint4 (&w)[BR / 4]) {
-    v = ldg16_if(live && colok, bl + (uint32_t)c * ldb);
+  // F32 blocks have no padding tiles: every tile of a full batch has a column
+  auto load_tile = [&](bool live, int64_t tt, int32_t c, uint4& v, uint4 (&w)[BR / 4]) {
+    if constexpr (FfmaShape<BR, G, FULL>::kReloadB)
+      v = ldg16_if(live && c >= 0 && colok, reinterpret_cast<const float*>(d.B) + (int64_t)c * d.ldb + n);
+    else if constexpr (PLAIN) v = ldg16_if(live, bl + (uint32_t)c * ldb);
+    else v = ldg16_if(live && c >= 0 && colok, Bp + (int64_t)c * d.ldb + n);
 #pragma unroll
     for (int r4 = 0; r4 < BR / 4; ++r4) w[r4] = ldg16_if(live, Av + tt * BR + r4 * 4);
+  };
+  auto load_full = [&](int64_t tt, int32_t c, uint4& v, uint4 (&w)[BR / 4]) {
+    if constexpr (PLAIN) {
+      v = ldg16(bl + (uint32_t)c * ldb);
+#pragma unroll
+      for (int r4 = 0; r4 < BR / 4; ++r4) w[r4] = ldg16(Av + tt * BR + r4 * 4);
+    } else {
+      load_tile(true, tt, c, v, w);
+    }
   };
   int32_t c[T];
   load_cols(t0, c);
@@ -323,7 +340,7 @@ __device__ __forceinline__ void ffma_unit(const BatchDesc& d, int64_t u, int sub
     uint4 v[T];
     uint4 w[T][BR / 4];
 #pragma unroll
-    for (int q = 0; q < T; ++q) load_tile(tt + q, c[q], v[q], w[q]);
+    for (int q = 0; q < T; ++q) load_full(tt + q, c[q], v[q], w[q]);
 #pragma unroll
     for (int q = 0; q < T; ++q) tile_fma(v[q], w[q]);
 #pragma unroll
@@ -333,7 +350,7 @@ __device__ __forceinline__ void ffma_unit(const BatchDesc& d, int64_t u, int sub
     uint4 v[T];
     uint4 w[T][BR / 4];
 #pragma unroll
-    for (int q = 0; q < T; ++q) load_tile_if(tt + q < t1, tt + q, c[q], v[q], w[q]);
+    for (int q = 0; q < T; ++q) load_tile(tt + q < t1, tt + q, c[q], v[q], w[q]);
 #pragma unroll
     for (int q = 0; q < T; ++q) tile_fma(v[q], w[q]);
   }
@@ -355,7 +372,7 @@ __device__ __forceinline__ void ffma_unit(const BatchDesc& d, int64_t u, int sub
 }
 
 template <int BR, int G, bool FULL>
-__global__ void __launch_bounds__(256, FfmaShape<BR>::kMinBlocks)
+__global__ void __launch_bounds__(256, (FfmaShape<BR, G, FULL>::kMinBlocks))
     batched_ffma(const BatchDesc* __restrict__ descs,
                                                        const BatchTask* __restrict__ tasks, int64_t n_tasks,
                                                        unsigned long long* counter) {
