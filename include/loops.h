@@ -18,9 +18,9 @@
  *    dimension (elements between consecutive rows), ld >= number of columns.
  *  - Every GPU call is ordered on the given stream (NULL = legacy default stream) and does
  *    not synchronise the device unless its comment says so.
- *  - A plan with split rows or split BCSR blocks (CSR rows above 512 entries with the default
- *    split_len: n_segments > 0; blocks above 256 tiles) keeps partial sums in its own device
- *    memory during loops_spmm and loops_spmm_backward: such calls on one plan must not overlap
+ *  - A plan with split rows or split BCSR blocks (n_segments > 0, with the default split_len only
+ *    where a CSR row is above 512 entries; blocks above 256 tiles) keeps partial sums in its own
+ *    device memory during loops_spmm and loops_spmm_backward: such calls on one plan must not overlap
  *    on the GPU. Calls on a plan without them may run on several streams at once.
  *  - Element types per plan dtype:
  *        dtype      A values stored   B, dC      C, dB, dvals   accumulation
@@ -104,7 +104,8 @@ typedef struct {
   int64_t r_boundary;
   int32_t want_backward;
   int32_t split_len;      /* CSR rows longer than this are split in segments of this length; 0 =
-                             default: rows above 512 entries, in segments of 64 to 512 by size */
+                             default: 64 to 512 by size where a row is above 512 entries, else none
+                             is split */
   int32_t tile_min;
   int32_t test_wide_maps; /* test hook: 64-bit value maps (loops_plan_set_values), which otherwise only
                              matrices of 2^31 entries or BCSR slots and more take; 0: by size */

@@ -302,8 +302,8 @@ _TORCH_OUT = {F64: "float64", F32: "float32", F16: "float32", BF16: "float32"}
 
 class Plan:
     """A LOOPS plan for C = A . B with B of N columns (``loops_plan``). Calls on one plan may overlap on
-    several streams unless it holds split rows (``info()["n_segments"]``; by default rows above 512
-    entries) or BCSR blocks above 256 tiles, whose partial sums are the plan's."""
+    several streams unless it holds split rows (``info()["n_segments"]``; by default where a row is above
+    512 entries) or BCSR blocks above 256 tiles, whose partial sums are the plan's."""
 
     def __init__(self, A, N: int, dtype: str = "f64", tau: float = 2.0, block_rows: int = 0,
                  want_backward: bool = False, contiguous_split: bool = False, r_boundary: int = 0,

@@ -22,11 +22,10 @@ constexpr int kCsrThreads = 128;
 constexpr int32_t kPastEnd = 1 << 30;  // an entry past every item's end
 
 // The long rows of a team launch, in three classes (longest first) of one team size each. They are the
-// items after the segments of cut rows, and the classes have the first blocks, in order.
+// first items (a set with teams has no cut rows), and the classes have the first blocks, in order.
 constexpr int kTeamMax = 8;     // groups
 constexpr int kTeamChunk = 32;  // entries
 struct Teams {
-  int32_t n_slots;
   int32_t n[3], log_size[3], block_end[3];
 };
 
@@ -53,8 +52,13 @@ struct CsrKArgs {
   double inv_scale_d;
   int64_t N;
   int accumulate;        // add to C (rows a BCSR part wrote first) instead of overwriting it
-  Teams team;            // team launches only
 };
+
+struct CsrTeamKArgs : CsrKArgs {
+  Teams team;
+};
+template <bool TEAMS>
+using LaunchArgs = std::conditional_t<TEAMS, CsrTeamKArgs, CsrKArgs>;
 
 template <class Tr>
 __device__ __forceinline__ typename Tr::TAcc out_scale(const CsrKArgs& a, int64_t n);
@@ -109,28 +113,33 @@ struct Share {
   int64_t item;
   int32_t first;     // entry
   int32_t skip;      // entries that the other groups take between two of its pieces
-  int32_t log_size;  // of the team; -1: one group
+  int32_t log_size;  // of the team
   bool live;
 };
-template <int G, bool TEAM>
-__device__ __forceinline__ Share share_of(const CsrKArgs& a) {
-  constexpr int kThreads = CsrBlock<G, TEAM>::kThreads;
-  if constexpr (TEAM) {
+// In a block of teams.
+template <int G>
+__device__ __forceinline__ Share team_share(const CsrTeamKArgs& a) {
+  constexpr int kThreads = CsrBlock<G, true>::kThreads;
+  const Teams& t = a.team;
+  const int b = (int)blockIdx.x, group = (int)threadIdx.x / G;
+  const int r = b < t.block_end[0] ? 0 : b < t.block_end[1] ? 1 : 2;
+  const int ls = t.log_size[r];
+  const int at = ((b - (r ? t.block_end[r - 1] : 0)) * (kThreads / G) + group) >> ls;
+  const bool live = at < t.n[r];  // the last block of a class may have teams without a row
+  const int before = (r > 0 ? t.n[0] : 0) + (r > 1 ? t.n[1] : 0);
+  return {(int64_t)before + (live ? at : 0), live ? (group & ((1 << ls) - 1)) * kTeamChunk : kPastEnd,
+          ((1 << ls) - 1) * kTeamChunk, ls, live};
+}
+// Elsewhere; TEAMS: in a launch that has team blocks.
+template <int G, bool TEAMS>
+__device__ __forceinline__ Share whole_item(const LaunchArgs<TEAMS>& a) {
+  constexpr int kThreads = CsrBlock<G, TEAMS>::kThreads;
+  if constexpr (TEAMS) {
     const Teams& t = a.team;
-    const int b = (int)blockIdx.x, group = (int)threadIdx.x / G;
-    if (b < t.block_end[2]) {
-      const int r = b < t.block_end[0] ? 0 : b < t.block_end[1] ? 1 : 2;
-      const int ls = t.log_size[r];
-      const int at = ((b - (r ? t.block_end[r - 1] : 0)) * (kThreads / G) + group) >> ls;
-      const bool live = at < t.n[r];  // the last block of a class may have teams without a row
-      const int before = (r > 0 ? t.n[0] : 0) + (r > 1 ? t.n[1] : 0);
-      return {(int64_t)t.n_slots + before + (live ? at : 0),
-              live ? (group & ((1 << ls) - 1)) * kTeamChunk : kPastEnd, ((1 << ls) - 1) * kTeamChunk, ls, live};
-    }
-    const int64_t g = (int64_t)(b - t.block_end[2]) * (kThreads / G) + group;
-    return {g < t.n_slots ? g : g + t.n[0] + t.n[1] + t.n[2], 0, 0, -1, true};
+    const int64_t g = (int64_t)((int)blockIdx.x - t.block_end[2]) * (kThreads / G) + (int)threadIdx.x / G;
+    return {g + t.n[0] + t.n[1] + t.n[2], 0, 0, 0, true};
   } else {
-    return {((int64_t)blockIdx.x * kThreads + threadIdx.x) / G, 0, 0, -1, true};
+    return {((int64_t)blockIdx.x * kThreads + threadIdx.x) / G, 0, 0, 0, true};
   }
 }
 
@@ -240,8 +249,7 @@ struct CsrShape {
 };
 
 template <class Tr, int G, int VPL, bool FULL, bool TEAM>
-__global__ void __launch_bounds__((CsrBlock<G, TEAM>::kThreads), (CsrShape<Tr, VPL>::kWarps * 32 / CsrBlock<G, TEAM>::kThreads))
-    csr_spmm_vec(CsrKArgs a) {
+__device__ __forceinline__ void spmm_vec_item(const CsrKArgs& a, const Share& sh) {
   using TB = typename Tr::TB;
   using TAcc = typename Tr::TAcc;
   using TV = typename Tr::TV;
@@ -253,7 +261,6 @@ __global__ void __launch_bounds__((CsrBlock<G, TEAM>::kThreads), (CsrShape<Tr, V
   static_assert(CH % U == 0, "load batches tile the chunk");
   const int lane = threadIdx.x & 31;
   const int sub = lane & (G - 1);
-  const Share sh = share_of<G, TEAM>(a);
   const int64_t item = sh.item;
   if (item >= a.n_items) return;  // a group leaves as a whole
   const unsigned gmask = (G == 32) ? 0xffffffffu : (((1u << G) - 1u) << (lane & ~(G - 1)));
@@ -323,9 +330,21 @@ __global__ void __launch_bounds__((CsrBlock<G, TEAM>::kThreads), (CsrShape<Tr, V
     }
   }
   if constexpr (TEAM) {
-    if (sh.log_size >= 0 && !team_sum<G>(sh, acc)) return;
+    if (!team_sum<G>(sh, acc)) return;
   }
   store_item<Tr, G, VPL>(a, row, n0, ok, acc);
+}
+
+template <class Tr, int G, int VPL, bool FULL, bool TEAMS>
+__global__ void __launch_bounds__((CsrBlock<G, TEAMS>::kThreads), (CsrShape<Tr, VPL>::kWarps * 32 / CsrBlock<G, TEAMS>::kThreads))
+    csr_spmm_vec(LaunchArgs<TEAMS> a) {
+  if constexpr (TEAMS) {
+    if ((int)blockIdx.x < a.team.block_end[2]) {
+      spmm_vec_item<Tr, G, VPL, FULL, true>(a, team_share<G>(a));
+      return;
+    }
+  }
+  spmm_vec_item<Tr, G, VPL, FULL, false>(a, whole_item<G, TEAMS>(a));
 }
 
 // Path for any N and alignment: a group of G lanes per item, each lane with CP pieces of VW adjacent
@@ -362,9 +381,7 @@ __device__ __forceinline__ void load_piece(bool on, const TB* p, TB (&x)[VW]) {
 }
 
 template <class Tr, int G, int CP, int VW, bool TEAM>
-__global__ void __launch_bounds__((CsrBlock<G, TEAM>::kThreads),
-                                  (TEAM && sizeof(typename Tr::TB) <= 4
-                                       ? OddShape<CP, VW>::kTeamWarps * 32 / CsrBlock<G, TEAM>::kThreads : 0)) csr_spmm_odd(CsrKArgs a) {
+__device__ __forceinline__ void spmm_odd_item(const CsrKArgs& a, const Share& sh) {
   using TB = typename Tr::TB;
   using TAcc = typename Tr::TAcc;
   using TC = typename Tr::TC;
@@ -373,7 +390,6 @@ __global__ void __launch_bounds__((CsrBlock<G, TEAM>::kThreads),
   static_assert(G % U == 0, "load batches tile the chunk of G entries");
   const int lane = threadIdx.x & 31;
   const int sub = lane & (G - 1);
-  const Share sh = share_of<G, TEAM>(a);
   const int64_t item = sh.item;
   if (item >= a.n_items) return;  // a group leaves as a whole
   const unsigned gmask = (G == 32) ? 0xffffffffu : (((1u << G) - 1u) << (lane & ~(G - 1)));
@@ -424,7 +440,7 @@ __global__ void __launch_bounds__((CsrBlock<G, TEAM>::kThreads),
     if (e0 < cnt) batch(e0, std::true_type());
   }
   if constexpr (TEAM) {
-    if (sh.log_size >= 0 && !team_sum<G>(sh, acc)) return;
+    if (!team_sum<G>(sh, acc)) return;
   }
 #pragma unroll
   for (int i = 0; i < CP; ++i) {
@@ -441,6 +457,20 @@ __global__ void __launch_bounds__((CsrBlock<G, TEAM>::kThreads),
       }
     }
   }
+}
+
+template <class Tr, int G, int CP, int VW>
+__global__ void __launch_bounds__(kCsrThreads) csr_spmm_odd(CsrKArgs a) {
+  spmm_odd_item<Tr, G, CP, VW, false>(a, whole_item<G, false>(a));
+}
+
+template <class Tr, int G, int CP, int VW>
+__global__ void __launch_bounds__((CsrBlock<G, true>::kThreads),
+                                  (sizeof(typename Tr::TB) <= 4
+                                       ? OddShape<CP, VW>::kTeamWarps * 32 / CsrBlock<G, true>::kThreads : 0))
+    csr_spmm_odd_teams(CsrTeamKArgs a) {
+  if ((int)blockIdx.x < a.team.block_end[2]) spmm_odd_item<Tr, G, CP, VW, true>(a, team_share<G>(a));
+  else spmm_odd_item<Tr, G, CP, VW, false>(a, whole_item<G, true>(a));
 }
 
 // C[row, n] = scale_n * sum over the row's segments, in segment order, eight partials in flight.
@@ -514,6 +544,7 @@ __device__ __noinline__ void weighted_dots(const int32_t* col, const int32_t* sr
                                            unsigned gmask, const typename Tr::TB* dC, int64_t lddc,
                                            const typename Tr::TB* Brow, const float* dc_scale, const float* b_scale,
                                            int64_t N, typename Tr::TC* dvals) {
+  __syncwarp(gmask);  // the caller's stores to dvals come before those that replace them
   for (int32_t k = sh.first; k < len; k = next_chunk<1, TEAM>(sh, k)) {
     const typename Tr::TB* drow = dC + (int64_t)col[k] * lddc;
     float s = 0.f;
@@ -527,8 +558,7 @@ __device__ __noinline__ void weighted_dots(const int32_t* col, const int32_t* sr
 }
 
 template <class Tr, int G, int VPL, bool FULL, bool TEAM>
-__global__ void __launch_bounds__((CsrBlock<G, TEAM>::kThreads), (BwdShape<Tr, VPL>::kWarps * 32 / CsrBlock<G, TEAM>::kThreads))
-    csr_backward_vec(CsrKArgs a, BwdKArgs w) {
+__device__ __forceinline__ void backward_item(const CsrKArgs& a, const BwdKArgs& w, const Share& sh) {
   using TB = typename Tr::TB;
   using TAcc = typename Tr::TAcc;
   using TC = typename Tr::TC;
@@ -540,7 +570,6 @@ __global__ void __launch_bounds__((CsrBlock<G, TEAM>::kThreads), (BwdShape<Tr, V
   static_assert(CH % U == 0, "load batches tile the chunk");
   const int lane = threadIdx.x & 31;
   const int sub = lane & (G - 1);
-  const Share sh = share_of<G, TEAM>(a);
   const int64_t item = sh.item;
   if (item >= a.n_items) return;  // a group leaves as a whole
   const unsigned gmask = (G == 32) ? 0xffffffffu : (((1u << G) - 1u) << (lane & ~(G - 1)));
@@ -685,18 +714,29 @@ __global__ void __launch_bounds__((CsrBlock<G, TEAM>::kThreads), (BwdShape<Tr, V
       }
     }
   }
+  bool holds = true;
+  if constexpr (TEAM) holds = team_sum<G>(sh, acc);
+  if (holds) store_item<Tr, G, VPL>(a, row, n0, ok, acc);
+  // after the accumulators' last use: live across the call they cost the whole step 9 % (GCN 2^18, N =
+  // 128, BF16: 637 -> 696 us)
   if constexpr (Tr::kScaled) {
-    if (__any_sync(gmask, lossy)) {
-      __syncwarp(gmask);  // the stores of the loop above come before those that replace them
+    if (__any_sync(gmask, lossy))
       weighted_dots<Tr, G, TEAM>(a.col + beg, w.src + beg, len, sh, sub, gmask, reinterpret_cast<const TB*>(a.B), a.ldb,
                                  reinterpret_cast<const TB*>(w.B) + (int64_t)j * w.ldb, w.dc_scale, w.b_scale, a.N,
                                  dvals);
+  }
+}
+
+template <class Tr, int G, int VPL, bool FULL, bool TEAMS>
+__global__ void __launch_bounds__((CsrBlock<G, TEAMS>::kThreads), (BwdShape<Tr, VPL>::kWarps * 32 / CsrBlock<G, TEAMS>::kThreads))
+    csr_backward_vec(LaunchArgs<TEAMS> a, BwdKArgs w) {
+  if constexpr (TEAMS) {
+    if ((int)blockIdx.x < a.team.block_end[2]) {
+      backward_item<Tr, G, VPL, FULL, true>(a, w, team_share<G>(a));
+      return;
     }
   }
-  if constexpr (TEAM) {
-    if (sh.log_size >= 0 && !team_sum<G>(sh, acc)) return;
-  }
-  store_item<Tr, G, VPL>(a, row, n0, ok, acc);
+  backward_item<Tr, G, VPL, FULL, false>(a, w, whole_item<G, TEAMS>(a));
 }
 
 inline int next_pow2(int64_t x) {
@@ -708,17 +748,18 @@ inline int next_pow2(int64_t x) {
 // Launches one of the three item kernels (`kernel` takes whether there are teams) over its items and
 // `chunks` column chunks.
 template <int G, class K>
-cudaError_t launch_items(CsrKArgs a, const CsrDev& d, int64_t chunks, K kernel) {
+cudaError_t launch_items(const CsrKArgs& args, const CsrDev& d, int64_t chunks, K kernel) {
   const int64_t team_rows = d.n_long[0] + d.n_long[1] + d.n_long[2];
   auto blocks_of = [](int64_t groups, int threads) { return (groups * G + threads - 1) / threads; };
   if (team_rows == 0) {
     constexpr int T = CsrBlock<G, false>::kThreads;
-    kernel(a, dim3((unsigned)blocks_of(a.n_items, T), (unsigned)chunks), T, std::false_type());
+    kernel(args, dim3((unsigned)blocks_of(args.n_items, T), (unsigned)chunks), T, std::false_type());
     return cudaGetLastError();
   }
   constexpr int T = CsrBlock<G, true>::kThreads;
+  CsrTeamKArgs a;
+  static_cast<CsrKArgs&>(a) = args;
   Teams& t = a.team;
-  t.n_slots = (int32_t)d.n_slots;
   int64_t blocks = 0;
   for (int r = 0; r < 3; ++r) {
     t.n[r] = (int32_t)d.n_long[r];
@@ -734,7 +775,7 @@ cudaError_t launch_items(CsrKArgs a, const CsrDev& d, int64_t chunks, K kernel) 
 template <class Tr, int G, int VPL>
 cudaError_t launch_vec_g(const CsrKArgs& a, const CsrDev& d, cudaStream_t s) {
   constexpr int64_t per_chunk = (int64_t)G * VPL * Tr::kVE;
-  return launch_items<G>(a, d, (a.N + per_chunk - 1) / per_chunk, [&](const CsrKArgs& k, dim3 grid, int threads, auto team) {
+  return launch_items<G>(a, d, (a.N + per_chunk - 1) / per_chunk, [&](const auto& k, dim3 grid, int threads, auto team) {
     constexpr bool T = decltype(team)::value;
     if (k.N % per_chunk == 0) csr_spmm_vec<Tr, G, VPL, true, T><<<grid, threads, 0, s>>>(k);
     else csr_spmm_vec<Tr, G, VPL, false, T><<<grid, threads, 0, s>>>(k);
@@ -746,8 +787,9 @@ cudaError_t launch_odd_vw(const CsrKArgs& a, const CsrDev& d, cudaStream_t s) {
   const int64_t pieces = a.N / VW;
   auto go = [&](auto g_tag, auto cp_tag) {
     constexpr int G = decltype(g_tag)::value, CP = decltype(cp_tag)::value;
-    return launch_items<G>(a, d, (pieces + G * CP - 1) / (G * CP), [&](const CsrKArgs& k, dim3 grid, int threads, auto team) {
-      csr_spmm_odd<Tr, G, CP, VW, decltype(team)::value><<<grid, threads, 0, s>>>(k);
+    return launch_items<G>(a, d, (pieces + G * CP - 1) / (G * CP), [&](const auto& k, dim3 grid, int threads, auto team) {
+      if constexpr (decltype(team)::value) csr_spmm_odd_teams<Tr, G, CP, VW><<<grid, threads, 0, s>>>(k);
+      else csr_spmm_odd<Tr, G, CP, VW><<<grid, threads, 0, s>>>(k);
     });
   };
   using std::integral_constant;
@@ -791,7 +833,6 @@ CsrKArgs csr_args(const loops_plan_s* p, const CsrDev& d, const DenseArgs& da, b
   a.inv_scale_f = da.inv_scale_f;
   a.inv_scale_d = da.inv_scale_d;
   a.N = da.N;
-  a.team = Teams();
   return a;
 }
 
@@ -848,9 +889,9 @@ cudaError_t launch_csr_backward_t(const CsrDev& d, const CsrKArgs& a, const BwdK
   auto go = [&](auto g_tag, auto p_tag) {
     constexpr int G = decltype(g_tag)::value;
     constexpr int VPL = decltype(p_tag)::value;
-    return launch_items<G>(a, d, 1, [&](const CsrKArgs& k, dim3 grid, int threads, auto team) {
+    return launch_items<G>(a, d, 1, [&](const auto& k, dim3 grid, int threads, auto team) {
       constexpr bool T = decltype(team)::value;
-      if (!T && k.N % (G * VPL * Tr::kVE) == 0) csr_backward_vec<Tr, G, VPL, !T, T><<<grid, threads, 0, s>>>(k, w);
+      if (k.N % (G * VPL * Tr::kVE) == 0) csr_backward_vec<Tr, G, VPL, true, T><<<grid, threads, 0, s>>>(k, w);
       else csr_backward_vec<Tr, G, VPL, false, T><<<grid, threads, 0, s>>>(k, w);
     });
   };

@@ -1,10 +1,10 @@
 // Device layout of a plan's two parts, and its inverse (export back to canonical order).
 //
-// CSR part: rows become work items processed in storage order; rows longer than cut_len
-// are cut into segments of split_len entries whose partial sums go to scratch slots and are summed afterwards in
-// slot order (deterministic). Items are ordered by decreasing length class, so the longest
-// work starts first (and the rows that a team may share follow the segments); within a class the
-// row order is kept.
+// CSR part: rows become work items processed in storage order. A set with a row longer than cut_len
+// has every row longer than split_len cut into segments of that length, whose partial sums go to
+// scratch slots and are summed afterwards in slot order (deterministic). Items are ordered by
+// decreasing length class, so the longest work starts first (the segments, or without them the rows
+// that a team may share); within a class the row order is kept.
 //
 // BCSR part: tile values are stored in the register-fragment order of the dtype's MMA, so a
 // lane loads its whole A fragment of a K-group with one vector load:
@@ -133,13 +133,19 @@ loops_status upload_part(loops_plan_s* p, int64_t N) {
     const int team_base = p->team_len > 0 ? bucket_of(p->team_len - 1) : -1;
     cd.team_len = p->team_len;
     int64_t n_slots = 0;
+    int64_t longest = 0;
+    for (int64_t x = 0; x < n_csr; ++x) {
+      const int mixed = in_bcsr.empty() ? 0 : in_bcsr[(size_t)c.csr_rows[(size_t)x]];
+      if (mixed == which) longest = std::max(longest, c.csr_ptr[(size_t)x + 1] - c.csr_ptr[(size_t)x]);
+    }
+    const int64_t cut = longest > p->cut_len ? L : p->cut_len;
     for (int64_t x = 0; x < n_csr; ++x) {
       const int32_t row = c.csr_rows[(size_t)x];
       const int mixed = in_bcsr.empty() ? 0 : in_bcsr[(size_t)row];
       if (mixed != which) continue;
       const int64_t b = c.csr_ptr[(size_t)x], e = c.csr_ptr[(size_t)x + 1];
       const int64_t len = e - b;
-      if (len > p->cut_len) {
+      if (len > cut) {
         cd.h_split_row.push_back(row);
         cd.h_split_slot_ptr.push_back((int32_t)n_slots);
         for (int64_t s0 = b; s0 < e; s0 += L) {
@@ -148,7 +154,7 @@ loops_status upload_part(loops_plan_s* p, int64_t N) {
         }
       } else {
         items.push_back({row, b, e, bucket_of(len)});
-        const int cls = long_class(items.back().bucket, team_base);
+        const int cls = longest > p->cut_len ? -1 : long_class(items.back().bucket, team_base);
         if (cls >= 0) ++cd.n_long[cls];
       }
     }

@@ -145,8 +145,8 @@ struct CsrDev {
   int32_t* split_row = nullptr;        // global C row of each split row
   int32_t* split_slot_ptr = nullptr;   // size n_split + 1
   void* scratch = nullptr;             // n_slots x N partial sums (accumulator type)
-  // uncut rows that a team of lane groups each takes, by class (long_class): the items after the
-  // segments, longest class first
+  // rows that a team of lane groups each takes, by class (long_class): the first items, longest class
+  // first (none where rows are cut)
   int64_t n_long[3] = {0, 0, 0};
   int32_t team_len = 0;
   void* slab = nullptr;                // when set, the one allocation that holds the arrays above
@@ -183,7 +183,7 @@ inline int long_class_log_team(int r, int32_t team_len) {
   return log;
 }
 
-// CSR rows longer than this are cut where the caller gives no split_len.
+// A CSR set with a row longer than this has its rows cut where the caller gives no split_len.
 constexpr int32_t kDefaultCutLen = 512;
 
 struct BcsrDev {
@@ -336,7 +336,7 @@ struct loops_plan_s {
   double tau;
   double scale;
   int32_t split_len;                   // length of the segments of a cut row (and of the SDDMM items)
-  int32_t cut_len;                     // rows longer than this are cut
+  int32_t cut_len;                     // with a row longer than this, rows longer than split_len are cut
   int32_t team_len;                    // uncut rows of about this length or more may have a team; 0: none
   int32_t tile_min;                    // tile-level split threshold in effect (0: off)
   loops_plan_opts opts;

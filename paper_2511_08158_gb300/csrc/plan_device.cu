@@ -684,7 +684,7 @@ __device__ __forceinline__ int bucket_of_len(int64_t len) {  // floor(log2(len +
 // Rows of one CSR set: set 0 takes every row of a CSR block (empty rows too; every row when
 // is_bcsr is null), set 1 the rows of BCSR blocks that have moved entries. Rows longer than `cut`
 // become split rows of ceil(len / L) segments; the uncut rows that a team may share are
-// counted by class (they follow the segments in the item order).
+// counted by class (they come first in the item order).
 struct RowSet {
   const int64_t* rp;
   const uint8_t* is_bcsr;
@@ -702,8 +702,12 @@ struct RowSet {
 // Work items, partial-sum slots, split rows and long uncut rows, of a row or summed.
 struct RowCount {
   int64_t items, slots, splits, longs[3];
+  int64_t fine_slots, fine_splits;  // with `cut` equal to L
   __device__ __forceinline__ void add(int64_t len, const RowSet& rs) {
-    const int64_t segs = len > rs.cut ? (len + rs.L - 1) / rs.L : 0;
+    const int64_t fine = len > rs.L ? (len + rs.L - 1) / rs.L : 0;
+    const int64_t segs = len > rs.cut ? fine : 0;
+    fine_slots += fine;
+    fine_splits += fine > 0;
     items += len < 0 ? 0 : (segs ? segs : 1);
     slots += segs;
     splits += segs > 0;
@@ -711,6 +715,13 @@ struct RowCount {
     const int cls = long_class(bucket_of_len(len), rs.team_base);
 #pragma unroll
     for (int r = 0; r < 3; ++r) longs[r] += cls == r;
+  }
+  // the counts with `cut` equal to L
+  __host__ __device__ __forceinline__ void refine() {
+    items += splits - slots + fine_slots - fine_splits;
+    slots = fine_slots;
+    splits = fine_splits;
+    for (int64_t& n : longs) n = 0;
   }
 };
 
@@ -726,6 +737,8 @@ __global__ void __launch_bounds__(kThreads) row_sums_k(RowSet rs, RowCount* sums
   block_excl_scan(c.items, tot.items);
   block_excl_scan(c.slots, tot.slots);
   block_excl_scan(c.splits, tot.splits);
+  block_excl_scan(c.fine_slots, tot.fine_slots);
+  block_excl_scan(c.fine_splits, tot.fine_splits);
   // at most kTile of each: the three together
   int64_t longs;
   block_excl_scan(c.longs[0] | c.longs[1] << 20 | c.longs[2] << 40, longs);
@@ -743,20 +756,24 @@ __global__ void __launch_bounds__(kThreads) row_sums_scan_k(RowCount* sums, int6
     at.items = carry.items + block_excl_scan(v.items, tot.items);
     at.slots = carry.slots + block_excl_scan(v.slots, tot.slots);
     at.splits = carry.splits + block_excl_scan(v.splits, tot.splits);
+    at.fine_slots = carry.fine_slots + block_excl_scan(v.fine_slots, tot.fine_slots);
+    at.fine_splits = carry.fine_splits + block_excl_scan(v.fine_splits, tot.fine_splits);
 #pragma unroll
     for (int r = 0; r < 3; ++r) at.longs[r] = carry.longs[r] + block_excl_scan(v.longs[r], tot.longs[r]);
     if (i < m) sums[i] = at;
     carry.items += tot.items;
     carry.slots += tot.slots;
     carry.splits += tot.splits;
+    carry.fine_slots += tot.fine_slots;
+    carry.fine_splits += tot.fine_splits;
 #pragma unroll
     for (int r = 0; r < 3; ++r) carry.longs[r] += tot.longs[r];
   }
   if (threadIdx.x == 0) sums[m] = carry;
 }
 
-// `total`: the totals of the scan, as read by the host.
-__global__ void __launch_bounds__(kThreads) row_emit_k(RowSet rs, const RowCount* sums, RowCount total,
+// `total`: the totals of the scan, as read by the host; refined: rs.cut has become L since the scan.
+__global__ void __launch_bounds__(kThreads) row_emit_k(RowSet rs, const RowCount* sums, RowCount total, bool refined,
                                                        const int64_t* cpos, uint64_t* ikey, int64_t* ival,
                                                        int32_t* pre_row, int64_t* pre_beg, int64_t* pre_len,
                                                        int32_t* split_row, int32_t* split_slot_ptr) {
@@ -770,6 +787,7 @@ __global__ void __launch_bounds__(kThreads) row_emit_k(RowSet rs, const RowCount
     c.add(lens[j], rs);
   }
   RowCount at = sums[blockIdx.x];
+  if (refined) at.refine();
   at.items += block_excl_scan(c.items, tot.items);
   at.slots += block_excl_scan(c.slots, tot.slots);
   at.splits += block_excl_scan(c.splits, tot.splits);
@@ -1024,7 +1042,7 @@ loops_status build_csr_set(loops_plan_s* p, const DevCsrIn& A, const int64_t* re
   const int64_t n = A.n_rows;
   if (n == 0) return LOOPS_OK;
   const int team_base = p->team_len > 0 ? bit_width((uint64_t)p->team_len) - 1 : -1;  // the class of team_len - 1
-  const RowSet rs{A.rp, is_bcsr, rowlen1, n, std::max<int64_t>(p->split_len, 1), std::max<int64_t>(p->cut_len, 1), p->br,
+  RowSet rs{A.rp, is_bcsr, rowlen1, n, std::max<int64_t>(p->split_len, 1), std::max<int64_t>(p->cut_len, 1), p->br,
                   which, team_base};
   const int64_t row_blocks = (n + kTile - 1) / kTile;
   RowCount* sums = ar.get<RowCount>(row_blocks + 1);
@@ -1034,6 +1052,11 @@ loops_status build_csr_set(loops_plan_s* p, const DevCsrIn& A, const int64_t* re
   TRY(cudaGetLastError());
   RowCount total{};
   TRY(to_host(&total, sums + row_blocks, s));
+  const bool refined = total.splits > 0 && rs.cut > rs.L;  // one row is cut: every row of the set above L is
+  if (refined) {
+    total.refine();
+    rs.cut = rs.L;
+  }
   const int64_t n_it = total.items;
   cd.n_items = n_it;
   cd.n_slots = total.slots;
@@ -1063,7 +1086,7 @@ loops_status build_csr_set(loops_plan_s* p, const DevCsrIn& A, const int64_t* re
   if (csr_src) slab.add((uint8_t**)csr_src, n_canon * (wide ? 8 : 4));
   TRY(slab.alloc(&cd.slab, bytes));
   if (csr_src) p->vmap.csr_src_in_slab = true;
-  row_emit_k<<<(unsigned)row_blocks, kThreads, 0, s>>>(rs, sums, total, cpos, ikey, ival, pre_row, pre_beg, pre_len,
+  row_emit_k<<<(unsigned)row_blocks, kThreads, 0, s>>>(rs, sums, total, refined, cpos, ikey, ival, pre_row, pre_beg, pre_len,
                                                        cd.split_row, cd.split_slot_ptr);
   TRY(cudaGetLastError());
   TRY(radix_sort<int64_t>(&ikey, &ival, &ikey2, &ival2, n_it, 6, ar, s));

@@ -1,6 +1,6 @@
 """Rows of up to 512 entries under the default split length: taken by a whole block where few of them
 would leave the chip idle, and without partial sums in the plan's memory, so that calls of one plan
-may overlap on two streams."""
+may overlap on two streams. With a longer row all are cut into segments."""
 import math
 
 import numpy as np
@@ -22,19 +22,20 @@ def rows_of(counts, n_cols, seed):
                           rng.standard_normal(rows.size), sort_cols=False)
 
 
-def skewed(seed):
-    """Short rows around rows at the edges of the length classes, the longest team rows and a cut row."""
+def skewed(seed, longest):
+    """Short rows around rows at the edges of the length classes and the longest team rows."""
     counts = np.arange(130) % 11
-    counts[3:120:9] = [62, 63, 64, 65, 126, 127, 128, 300, 511, 512, 513, 700, 100]
+    counts[3:120:9] = [62, 63, 64, 65, 126, 127, 128, 300, 511, 512, longest, 400, 100]
     return rows_of(counts, 140, seed)
 
 
 @pytest.mark.parametrize("fmt", ["f64", "f32", "f16", "bf16"])
+@pytest.mark.parametrize("longest,cut_rows", [(512, 0), (513, 10)])      # segments of 64
 @pytest.mark.parametrize("N", [1, 2, 4, 8, 13, 16, 26, 32, 47, 64, 66, 97, 128, 136, 194, 256, 520])
-def test_long_rows(loops_lib, fmt, N):
+def test_long_rows(loops_lib, fmt, N, longest, cut_rows):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
-    A = skewed(N)
+    A = skewed(N, longest)
     A_r, Bg, s, B_eff = rounded_inputs(A, W.dense_normal(140, N, N + 1), fmt)
     cs = torch.as_tensor(s, dtype=torch.float32).cuda() if s is not None else None
     dCq = oracle.round_to(W.dense_normal(A.n_rows, N, 2), fmt)
@@ -42,7 +43,7 @@ def test_long_rows(loops_lib, fmt, N):
     out = []
     for on_device in (False, True):
         plan = loops_lib.Plan(A, N, fmt, tau=math.inf, want_backward=True, build_on_device=on_device)
-        assert plan.info()["n_split_rows"] == 2              # 513 and 700 entries
+        assert plan.info()["n_split_rows"] == cut_rows
         C = plan.spmm(to_device(torch, Bg, fmt, ld=N + 8), col_scale=cs)
         dB, dv = plan.backward(to_device(torch, dCq, fmt), to_device(torch, Bq, fmt))
         assert rel_l2(C.double().cpu().numpy(), oracle.spmm(A_r, B_eff)) <= TOL[fmt]
