@@ -30,8 +30,8 @@
  *        LOOPS_BF16 bf16 (x s_A)      bf16       f32            f32 (HMMA)
  *    s_A is a power-of-two plan scale (max|a| * s_A <= 2^14) that the epilogue divides out
  *    exactly; the 16-bit dense operands may carry per-column power-of-two scales.
- *  - Inputs must be finite: a zero slot of a BCSR tile multiplies its B row, and 0 * inf
- *    is NaN under IEEE 754.
+ *  - Inputs must be finite: a zero slot of an F32, F16 or BF16 BCSR tile multiplies its B row, and
+ *    0 * inf is NaN under IEEE 754. F64 tiles skip their zeros, explicit zeros of A among them.
  */
 #ifndef LOOPS_H
 #define LOOPS_H

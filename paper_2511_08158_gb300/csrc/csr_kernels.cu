@@ -54,6 +54,8 @@ struct CsrKArgs {
   int accumulate;        // add to C (rows a BCSR part wrote first) instead of overwriting it
 };
 
+// Launches without teams do not take these: as part of CsrKArgs they changed the compiled loops of some kernels
+// (200,003-node graph, N = 97, FP32: 8 % slower; small graphs 15 %).
 struct CsrTeamKArgs : CsrKArgs {
   Teams team;
 };
@@ -239,7 +241,8 @@ __device__ __forceinline__ void store_item(const CsrKArgs& a, int32_t row, int32
 // * Columns in slices that fit L2 (64 to 512 bytes of each row at a time) were 2 to 40 % slower:
 //   the entries are read once per slice, and shorter pieces cost more instructions per byte.
 // FP64 is bound by the FP64 pipe: one entry at a time, so that no FMA is spent on a padded slot,
-// and no entries ahead; 48 warps per SM with one vector per lane (at 64 its 32 registers spill).
+// and no entries ahead; 48 warps per SM with one vector per lane (40 registers; instances of 1 and 32 lanes
+// spill 4 to 36 bytes). At 64 warps its 32 registers spill 8, and the time is the same within 2 %.
 template <class Tr, int VPL>
 struct CsrShape {
   static constexpr bool kF64 = std::is_same<Tr, TrF64>::value;
@@ -352,8 +355,8 @@ __global__ void __launch_bounds__((CsrBlock<G, TEAMS>::kThreads), (CsrShape<Tr, 
 // reads consecutive memory and a row of B in one pass. With loads of 2 to 8 bytes instructions
 // count first: few lanes with many pieces each (G = 8 up to 64 pieces per row) share an entry's
 // column, value and address over CP loads, waste few lanes on a ragged N, and let a warp take
-// several items. U entries with 8 to 24 elements in flight per lane, entries one chunk ahead.
-// 200,003-node graph, 4.1 M entries, N = 47, FP32: @ODD@, against 280 us with one column per lane
+// several items. U entries with 8 to 32 elements in flight per lane, entries one chunk ahead.
+// 200,003-node graph, 4.1 M entries, N = 47, FP32: 100 us, against 280 us with one column per lane
 // and the entries read per 32 columns, and 165 us with 32 lanes and two pieces.
 template <int CP, int VW>
 struct OddShape {
@@ -509,11 +512,14 @@ __global__ void __launch_bounds__(kReduceThreads) split_reduce(const int32_t* __
 // it gathers. The gathers of dC rows bound it as they bound the SpMM and the SDDMM that it
 // replaces, and are made once instead of twice. Measured on GB300 (dB and dvals together):
 //   GCN 2^18, 7.4 M entries, N = 256, FP32      930 -> 566 us
-//   the same graph, N = 128, BF16               369 -> 265 us
+//   the same graph, N = 128, BF16               369 -> 265 us (about 4 us more with the check of the weights)
 // The shape is the SpMM's: 128 threads, entries one chunk ahead, no predicates where the group
 // covers the columns. Bytes in flight and warps decide: FP32 takes four entries in flight at 32
 // warps per SM (two: 10 % slower step; 24 warps: 5 %), the 16-bit formats two vectors per lane
-// from 16 on with two entries at 28 warps (one vector: 4 % slower step; 32 warps spill: 11 %).
+// from 16 on with two entries at 28 warps (one vector: 4 % slower step; 32 warps spill: 11 %). Other instances
+// spill: partly covered FP32 with two vectors 72 to 92 bytes, one lane per row (N of one vector) 130 to 230. Against
+// the two kernels they are still ahead: 100,000 nodes, 1.7 M entries, FP32 N = 4 726 -> 53 us, 36 179 -> 57, 136
+// 340 -> 176; BF16 N = 8 758 -> 74; FP64 N = 2 333 -> 69, 72 935 -> 923.
 // The input entry of a dot product (`src`) is loaded with its column and value: loaded where
 // dvals is stored, it stalled every batch (20 % slower).
 template <class Tr, int VPL>
@@ -717,8 +723,7 @@ __device__ __forceinline__ void backward_item(const CsrKArgs& a, const BwdKArgs&
   bool holds = true;
   if constexpr (TEAM) holds = team_sum<G>(sh, acc);
   if (holds) store_item<Tr, G, VPL>(a, row, n0, ok, acc);
-  // after the accumulators' last use: live across the call they cost the whole step 9 % (GCN 2^18, N =
-  // 128, BF16: 637 -> 696 us)
+  // after the accumulators' last use, so that none is live across the call
   if constexpr (Tr::kScaled) {
     if (__any_sync(gmask, lossy))
       weighted_dots<Tr, G, TEAM>(a.col + beg, w.src + beg, len, sh, sub, gmask, reinterpret_cast<const TB*>(a.B), a.ldb,
